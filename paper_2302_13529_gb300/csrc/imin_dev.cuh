@@ -215,7 +215,9 @@ struct CtaCfg {
                              // by list position after the grid's slots (Handoff below)
     uint64_t off_bm, off_gid, off_par, off_idom, off_rows, off_edges, slot_bytes;
     uint8_t* scratch;
-    uint32_t from_list;   // 1: take the samples that tier 0 handed over; 0: all of [0, theta)
+    uint32_t from_list;   // 1: take the samples listed for in_tier; 0: all of [0, theta)
+    uint32_t in_tier;     // tier whose work cursor and sample list the launch uses (kTierCta)
+    uint32_t out_tier;    // tier whose list receives the samples that do not fit (kTierWhole)
 };
 
 // One query of a batch (batch.cu): its graph, seed set, masks, counters and results.

@@ -79,6 +79,11 @@ struct TierPlan {
 // Capacities and per-warp shared-memory bytes of the warp tier 0 (working set in shared memory)
 // for seed sets of up to ns vertices and r0 non-seed vertices.
 void tier0_cfg(uint32_t ns, uint32_t r0, TierCfg* c);
+// The warp tier 0 in front of a block tier, for callers that must not query the runtime on each
+// call: capacities, grid and shared memory from the sizes alone (blocks 0: the seed set does not
+// fit). allow_tier0_smem must have run once on the device.
+void plan_tier0(const DeviceInfo& dev, uint32_t ns, uint32_t cutoff, TierPlan* p);
+void allow_tier0_smem(const DeviceInfo& dev);
 // cutoff: non-seed capacity of the warp tier 0 run in front of the block tier (0: none).
 TierPlan plan_tiers(const DeviceInfo& dev, int32_t n, int32_t m, uint32_t ns, uint32_t cutoff);
 
@@ -92,6 +97,8 @@ cudaError_t launch_sample_tier(int tier, const SampleParams& P, const TierPlan& 
 
 // Block-per-sample tier: layout, grid and shared memory. Graphs with n <= kCtaMaxVertices keep
 // the visited bitmap in shared memory; larger ones keep it in each block's global slot.
+// Offsets and size of a block's slot, from c's capacities (rcap, ecap) and bitmap size.
+void cta_slot_layout(CtaCfg* c);
 bool plan_cta_tier(const DeviceInfo& dev, int32_t n, int32_t m, CtaCfg* c, uint32_t* blocks, uint64_t* smem,
                    uint64_t* scratch_bytes);
 cudaError_t launch_cta_tier(const SampleParams& P, const CtaCfg& c, uint32_t blocks, uint64_t smem,

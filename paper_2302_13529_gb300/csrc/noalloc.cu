@@ -8,8 +8,8 @@
 // its kernel runs and the kernel's status after it, so it returns only when the counters are
 // final, and it cannot be recorded into a CUDA graph by stream capture.
 //
-// What it does: exactly what imin_estimate_decrease computes, with the block-per-sample tier
-// (sample_cta.cu), but every byte of working memory it needs besides the caller's inputs and
+// What it does: exactly what imin_estimate_decrease computes, with the warp tier at a fixed cutoff
+// (sample.cu) in front of the block-per-sample tier (sample_cta.cu), but every byte of working memory it needs besides the caller's inputs and
 // output comes from one file-scope device array of kNoAllocBytes (64 MiB). Every GPU that loads
 // the library holds that array until the process exits. Its limits follow from its size:
 // graphs with at most kNoAllocMaxVertices vertices and at most kNoAllocMaxTheta samples per call;
@@ -28,6 +28,7 @@
 // once per device and graph size (n, m) and kept in a fixed table, so later calls of the same
 // size make no attribute or occupancy queries; the plan's test hooks (IMIN_CTA_EDGE_CAP) are read
 // only when a plan is made.
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -57,6 +58,10 @@ struct PlanEntry {
     uint32_t blocks;
     uint64_t smem;
 };
+// Slot capacities of the first block-tier launch (vertices, non-tree edges): the smallest that hold
+// all but the rare cascades, so that a slot for every resident block (8 per SM) fits the array.
+constexpr uint32_t kSmallVertices = 2048;
+constexpr uint32_t kSmallEdges = 1024;
 constexpr int kPlanSlots = 16;
 PlanEntry g_plans[kPlanSlots];
 int g_plan_count = 0, g_plan_next = 0;
@@ -76,6 +81,7 @@ bool cta_plan(const imin_graph* g, CtaCfg* cfg, uint32_t* blocks, uint64_t* smem
     }
     uint64_t slot_total = 0;
     if (!plan_cta_tier(g->dev, g->n, g->m, cfg, blocks, smem, &slot_total)) return false;
+    allow_tier0_smem(g->dev);
     PlanEntry& e = g_plans[g_plan_next];
     e = PlanEntry{g->device, g->n, g->m, *cfg, *blocks, *smem};
     g_plan_next = (g_plan_next + 1) % kPlanSlots;
@@ -211,8 +217,21 @@ extern "C" int imin_estimate_decrease_noalloc(const imin_graph* g, const int32_t
         return fail_msg(IMIN_ERR_INTERNAL, "the block-per-sample kernel cannot be configured");
     if (off_slots + cfg.slot_bytes > kNoAllocBytes)
         return fail_msg(IMIN_ERR_INVALID, "imin_estimate_decrease_noalloc: request exceeds the static scratch");
-    const uint64_t slots = (kNoAllocBytes - off_slots) / cfg.slot_bytes;
-    if (slots < blocks) blocks = static_cast<uint32_t>(slots);
+    const uint64_t room = kNoAllocBytes - off_slots;
+    // Whole-graph slots are so large that few fit (56 at n = 50,000, where 1,216 blocks could be
+    // resident). So a call has up to three launches: the warp tier, which needs no slots; the block
+    // tier on slots of kSmallVertices, one per resident block; and the block tier on whole-graph
+    // slots for the samples that outgrow those. The launches follow one another on the stream and
+    // share the array. n = 50,021, m = 400,009, theta = 10^4, |S| = 50: 6.26 -> 2.40 ms. The second
+    // launch must read the first's overflow count either way, so it is always enqueued.
+    CtaCfg small = cfg;
+    small.rcap = std::min(cfg.rcap, std::max(kSmallVertices, 2u * (1u + static_cast<uint32_t>(n_seeds))));
+    small.ecap = std::min(cfg.ecap, kSmallEdges);
+    cta_slot_layout(&small);
+    const uint32_t small_blocks = static_cast<uint32_t>(std::min<uint64_t>(blocks, room / small.slot_bytes));
+    const uint32_t whole_blocks = static_cast<uint32_t>(std::min<uint64_t>(blocks, room / cfg.slot_bytes));
+    TierPlan warp{};
+    plan_tier0(g->dev, static_cast<uint32_t>(n_seeds), kDefaultCutoff, &warp);
 
     RoundCtl* ctl = reinterpret_cast<RoundCtl*>(base + off_ctl);
     uint32_t* bad = reinterpret_cast<uint32_t*>(base + off_bad);
@@ -252,7 +271,14 @@ extern "C" int imin_estimate_decrease_noalloc(const imin_graph* g, const int32_t
     P.lists = reinterpret_cast<uint32_t*>(base + off_lists);
     P.done = nullptr;
     P.stats = nullptr;
-    NA_CUDA(launch_cta_tier(P, cfg, blocks, smem, base + off_slots, s));
+    bool warp_ran = false;
+    NA_CUDA(launch_sample_tier(0, P, warp, nullptr, s, &warp_ran));
+    small.from_list = warp_ran ? 1u : 0u;
+    NA_CUDA(launch_cta_tier(P, small, small_blocks, smem, base + off_slots, s));
+    cfg.from_list = 1;
+    cfg.in_tier = kTierWhole;
+    cfg.out_tier = 1;  // the warp tier 1 does not run here: its list takes what nothing here holds
+    NA_CUDA(launch_cta_tier(P, cfg, whole_blocks, smem, base + off_slots, s));
 
     RoundCtl hctl;
     NA_CUDA(cudaMemcpyAsync(&hctl, ctl, sizeof(hctl), cudaMemcpyDeviceToHost, s));
@@ -260,7 +286,7 @@ extern "C" int imin_estimate_decrease_noalloc(const imin_graph* g, const int32_t
         NA_CUDA(cudaMemcpyAsync(out_delta, delta, 8ull * g->n, cudaMemcpyDeviceToHost, s));
     NA_CUDA(cudaStreamSynchronize(s));
     if (hctl.error & kErrInternal) return fail_msg(IMIN_ERR_INTERNAL, "dominator iteration did not converge");
-    if (hctl.count[kTierWhole] > 0)
+    if (hctl.count[1] > 0)
         return fail_msg(IMIN_ERR_CAPACITY,
                         "imin_estimate_decrease_noalloc: a sampled cascade needs the whole-graph "
                         "tier, which this entry point does not run");

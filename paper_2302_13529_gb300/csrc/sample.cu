@@ -162,6 +162,23 @@ void tier0_cfg(uint32_t ns, uint32_t r0, TierCfg* c)
     c->next_tier = kTierCta;
 }
 
+void allow_tier0_smem(const DeviceInfo& dev)
+{
+    allow_max_dynamic_smem(k_sample_tier<0, kModelLT>, dev);
+    allow_max_dynamic_smem(k_sample_tier<0, kModelIC>, dev);
+}
+
+void plan_tier0(const DeviceInfo& dev, uint32_t ns, uint32_t cutoff, TierPlan* p)
+{
+    tier0_cfg(ns, cutoff, &p->cfg[0]);
+    p->warps_per_block[0] = kWarpsPerBlock;
+    p->smem_bytes[0] = kWarpsPerBlock * (kStageBytes + p->cfg[0].warp_bytes);
+    p->scratch_bytes[0] = 0;
+    // 5 blocks of 48 registers a thread share an SM; blocks that do not fit at once find the work
+    // cursor where the resident ones left it
+    p->blocks[0] = p->smem_bytes[0] <= dev.smem_optin ? 5u * dev.sms : 0u;
+}
+
 TierPlan plan_tiers(const DeviceInfo& dev, int32_t n, int32_t m, uint32_t ns, uint32_t cutoff)
 {
     TierPlan p{};
@@ -192,8 +209,7 @@ TierPlan plan_tiers(const DeviceInfo& dev, int32_t n, int32_t m, uint32_t ns, ui
         p.scratch_bytes[0] = 0;
         int occ = 0;
         if (p.smem_bytes[0] <= dev.smem_optin) {
-            allow_max_dynamic_smem(k_sample_tier<0, kModelLT>, dev);
-            allow_max_dynamic_smem(k_sample_tier<0, kModelIC>, dev);
+            allow_tier0_smem(dev);
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sample_tier<0, kModelIC>,
                                                           kWarpsPerBlock * 32, p.smem_bytes[0]);
         }

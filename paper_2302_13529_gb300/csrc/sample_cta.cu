@@ -44,12 +44,12 @@ __global__ void __launch_bounds__(cta_threads<kSmemBitmap>(), 1024 / cta_threads
     unsigned long long examined = 0, live = 0;
     for (;;) {
         __syncthreads();
-        if (tid == 0) sh.item = atomicAdd(&P.ctl->cursor[kTierCta], 1u);
+        if (tid == 0) sh.item = atomicAdd(&P.ctl->cursor[C.in_tier], 1u);
         __syncthreads();
         const uint32_t total =
-            C.from_list ? *reinterpret_cast<const volatile uint32_t*>(&P.ctl->count[kTierCta]) : P.theta;
+            C.from_list ? *reinterpret_cast<const volatile uint32_t*>(&P.ctl->count[C.in_tier]) : P.theta;
         if (sh.item >= total) break;
-        const uint32_t j = C.from_list ? P.lists[kTierCta * P.theta + sh.item] : sh.item;
+        const uint32_t j = C.from_list ? P.lists[C.in_tier * P.theta + sh.item] : sh.item;
         int rc;
         if (C.handoff_stride != 0) {
             // the warp tier left this sample's state at the level it could not hold: resume there
@@ -64,8 +64,8 @@ __global__ void __launch_bounds__(cta_threads<kSmemBitmap>(), 1024 / cta_threads
         }
         if (tid == 0) {
             if (rc == kSampleOverflow) {
-                const uint32_t pos = atomicAdd(&P.ctl->count[kTierWhole], 1u);
-                P.lists[kTierWhole * P.theta + pos] = j;
+                const uint32_t pos = atomicAdd(&P.ctl->count[C.out_tier], 1u);
+                P.lists[C.out_tier * P.theta + pos] = j;
             } else if (rc == kSampleError) {
                 atomicOr(&P.ctl->error, kErrInternal);
             }
@@ -97,6 +97,18 @@ __global__ void __launch_bounds__(cta_threads<kSmemBitmap>(), 1024 / cta_threads
 
 }  // namespace
 
+void cta_slot_layout(CtaCfg* c)
+{
+    uint64_t o = 0;
+    c->off_bm = o;    o = align16(o + (c->global_bitmap ? 4ull * c->bm_words : 0ull));
+    c->off_gid = o;   o = align16(o + 4ull * c->rcap);
+    c->off_par = o;   o = align16(o + 4ull * c->rcap);
+    c->off_idom = o;  o = align16(o + 4ull * c->rcap);
+    c->off_rows = o;  o = align16(o + 8ull * c->rcap);
+    c->off_edges = o; o = align16(o + 8ull * c->ecap);
+    c->slot_bytes = (o + 255) & ~255ull;
+}
+
 bool plan_cta_tier(const DeviceInfo& dev, int32_t n, int32_t m, CtaCfg* c, uint32_t* blocks, uint64_t* smem,
                    uint64_t* scratch_bytes)
 {
@@ -112,6 +124,8 @@ bool plan_cta_tier(const DeviceInfo& dev, int32_t n, int32_t m, CtaCfg* c, uint3
     }
     c->global_bitmap = smem_bitmap ? 0u : 1u;
     c->handoff_stride = 0;  // set per query when the warp tier runs in front (api.cu)
+    c->in_tier = kTierCta;
+    c->out_tier = kTierWhole;
     c->tree_words = smem_bitmap ? c->bm_words : 2 * slots;
     c->res_slots = slots;
     uint32_t bits = 0;
@@ -132,14 +146,7 @@ bool plan_cta_tier(const DeviceInfo& dev, int32_t n, int32_t m, CtaCfg* c, uint3
         const uint32_t v = static_cast<uint32_t>(std::strtoul(cap, nullptr, 10));
         if (v > 0) c->rcap = std::max<uint32_t>(std::min(c->rcap, v), 2u);
     }
-    uint64_t o = 0;
-    c->off_bm = o;    o = align16(o + (smem_bitmap ? 0ull : 4ull * c->bm_words));
-    c->off_gid = o;   o = align16(o + 4ull * c->rcap);
-    c->off_par = o;   o = align16(o + 4ull * c->rcap);
-    c->off_idom = o;  o = align16(o + 4ull * c->rcap);
-    c->off_rows = o;  o = align16(o + 8ull * c->rcap);
-    c->off_edges = o; o = align16(o + 8ull * c->ecap);
-    c->slot_bytes = (o + 255) & ~255ull;
+    cta_slot_layout(c);
     *smem = smem_bitmap ? 4ull * c->bm_words : 8ull * slots;
     if (*smem > dev.smem_optin) return false;
     int occ = 0;
