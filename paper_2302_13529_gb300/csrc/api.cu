@@ -331,6 +331,22 @@ cudaError_t enqueue_call(const SampleParams& P, const Query& q, CallTimer& T)
     return cudaSuccess;
 }
 
+// All slices of a spread call (spread.cu): the warp kernel and the block kernel of each.
+cudaError_t enqueue_spread(const SampleParams& P, const Query& q, CallTimer& T, const int32_t* sets, uint32_t k,
+                           unsigned long long items, uint32_t* handoff, unsigned long long* sums)
+{
+    for (unsigned long long i = 0; i < spread_slices(items); ++i) {
+        const cudaError_t e = T.run(kKindCta, [&](bool* launched) {
+            *launched = true;
+            g_launches.fetch_add(1, std::memory_order_relaxed);  // the slice's second kernel
+            return launch_spread_slice(P, q.plan.cta, q.plan.blocks[kTierCta], q.plan.smem_bytes[kTierCta],
+                                       q.scratch3, sets, k, items, i, handoff, sums, T.s);
+        });
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 cudaError_t enqueue_select(const SelectParams& sp, CallTimer& T)
 {
     return T.run(kKindSelect, [&](bool* launched) {
@@ -670,6 +686,8 @@ int spread_impl(const imin_graph* g, const int32_t* seeds, int32_t n_seeds, cons
     RoundCtl* ctl = nullptr;
     int32_t* dblocked = nullptr;
     unsigned long long* dsum = nullptr;
+    uint32_t* handoff = nullptr;
+    IMIN_CUDA(q.arena.alloc(&handoff, spread_handoff_words(theta)));
     IMIN_CUDA(q.arena.alloc(&ctl, 1));
     IMIN_CUDA(q.arena.alloc(&dblocked, hblocked.size()));
     IMIN_CUDA(q.arena.alloc(&dsum, 1));
@@ -683,11 +701,7 @@ int spread_impl(const imin_graph* g, const int32_t* seeds, int32_t n_seeds, cons
     }
     CallTimer T(s);
     const SampleParams P = sample_params(g, q, static_cast<uint32_t>(n_seeds), theta, key, round, ctl, nullptr);
-    IMIN_CUDA(T.run(kKindCta, [&](bool* launched) {
-        *launched = true;
-        return launch_spread(P, q.plan.cta, q.plan.blocks[kTierCta], q.plan.smem_bytes[kTierCta], q.scratch3,
-                             dsum, s);
-    }));
+    IMIN_CUDA(enqueue_spread(P, q, T, nullptr, 0, theta, handoff, dsum));
     std::vector<RoundCtl> hctl(1);
     unsigned long long hstats[kStCount], hsum = 0;
     IMIN_CUDA(cudaMemcpyAsync(hctl.data(), ctl, sizeof(RoundCtl), cudaMemcpyDeviceToHost, s));
@@ -740,15 +754,15 @@ int spread_sets_core(const imin_graph* g, const std::vector<int32_t>& hseeds, co
     int32_t* dblocked = nullptr;
     int32_t* dsets = nullptr;
     unsigned long long* dsums = nullptr;
-    unsigned long long* cursor = nullptr;
+    uint32_t* handoff = nullptr;
+    const unsigned long long items = static_cast<unsigned long long>(nsets) * theta;
     IMIN_CUDA(q.arena.alloc(&ctl, 1));
     IMIN_CUDA(q.arena.alloc(&dblocked, hblocked.size()));
     IMIN_CUDA(q.arena.alloc(&dsets, static_cast<uint64_t>(nsets) * k));
     IMIN_CUDA(q.arena.alloc(&dsums, static_cast<uint64_t>(nsets)));
-    IMIN_CUDA(q.arena.alloc(&cursor, 1));
+    IMIN_CUDA(q.arena.alloc(&handoff, spread_handoff_words(items)));
     IMIN_CUDA(cudaMemsetAsync(ctl, 0, sizeof(RoundCtl), s));
     IMIN_CUDA(cudaMemsetAsync(dsums, 0, sizeof(unsigned long long) * nsets, s));
-    IMIN_CUDA(cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), s));
     if (k > 0)
         IMIN_CUDA(cudaMemcpyAsync(dsets, hsets, sizeof(int32_t) * nsets * k, cudaMemcpyHostToDevice, s));
     if (!hblocked.empty()) {
@@ -758,13 +772,9 @@ int spread_sets_core(const imin_graph* g, const std::vector<int32_t>& hseeds, co
         g_launches.fetch_add(1, std::memory_order_relaxed);
     }
     CallTimer T(s);
-    const SampleParams P = sample_params(g, q, static_cast<uint32_t>(hseeds.size()), theta, key, round, ctl, nullptr);
-    IMIN_CUDA(T.run(kKindCta, [&](bool* launched) {
-        *launched = true;
-        return launch_spread_sets(P, q.plan.cta, q.plan.blocks[kTierCta], q.plan.smem_bytes[kTierCta], q.scratch3,
-                                  dsets, static_cast<uint32_t>(k),
-                                  static_cast<unsigned long long>(nsets) * theta, cursor, dsums, s);
-    }));
+    SampleParams P = sample_params(g, q, static_cast<uint32_t>(hseeds.size()), theta, key, round, ctl, nullptr);
+    P.stats = nullptr;
+    IMIN_CUDA(enqueue_spread(P, q, T, dsets, static_cast<uint32_t>(k), items, handoff, dsums));
     RoundCtl hctl;
     IMIN_CUDA(cudaMemcpyAsync(&hctl, ctl, sizeof(hctl), cudaMemcpyDeviceToHost, s));
     IMIN_CUDA(cudaMemcpyAsync(hsums, dsums, sizeof(uint64_t) * nsets, cudaMemcpyDeviceToHost, s));
@@ -1078,6 +1088,7 @@ int batch_impl(Driver which, imin_query* qs, int32_t nq, void* stream, uint32_t 
     if (global_bytes > 0)
         IMIN_CUDA(prepare_cta_scratch(cfg[kBatchGlobalClass], cta_blocks[kBatchGlobalClass], global_scratch, s));
     IMIN_CUDA(arena.alloc(&whole_scratch, wp.scratch_bytes[kTierWhole]));
+    IMIN_CUDA(cudaMemsetAsync(whole_scratch, 0xFF, wp.scratch_bytes[kTierWhole], s));
     IMIN_CUDA(arena.alloc(&stats, kStCount));
     // hand-off snapshots of the samples the warp tier gives up on, per size class after the
     // overflow items (at most 1 GiB in all; samples beyond the lists' room run from the start)
@@ -1098,7 +1109,6 @@ int batch_impl(Driver which, imin_query* qs, int32_t nq, void* stream, uint32_t 
     over = reinterpret_cast<uint2*>(over_raw);
     IMIN_CUDA(arena.alloc(&cb_counts, nq));
     IMIN_CUDA(cudaMemsetAsync(buf, 0, total, s));
-    IMIN_CUDA(cudaMemsetAsync(whole_scratch, 0xFF, wp.scratch_bytes[kTierWhole], s));
     IMIN_CUDA(cudaMemsetAsync(stats, 0, sizeof(unsigned long long) * kStCount, s));
     IMIN_CUDA(cudaMemsetAsync(cb_counts, 0, sizeof(uint32_t) * nq, s));
     std::vector<int32_t> hseed_all(seed_off[nq]);

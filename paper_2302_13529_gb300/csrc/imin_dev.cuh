@@ -310,6 +310,99 @@ __host__ __device__ inline WarpLayout warp_layout(uint32_t rcap, uint32_t hcap, 
     return L;
 }
 
+// Shared-memory work area of one warp's frontier chunk (always shared memory).
+// The non-empty rows of up to 32 frontier vertices, in order, and the live edges that wait to be
+// visited: at most 31 left over plus one iteration's 32 lanes x 4 edges.
+constexpr uint32_t kLiveCap = 160;
+struct __align__(16) WarpStage {
+    uint32_t edge[kLiveCap];  // live edge ids
+    int32_t beg[32], end[32];  // edge range of each non-empty row
+    uint32_t qoff[32];         // the row's 4-edge group of flat index t is qoff + t
+    uint8_t vert[32];          // the row's vertex: its position in the chunk
+    uint8_t src[kLiveCap];    // the staged edge's row
+};
+
+// The flattened 4-edge groups of a chunk: a lane's own row starts at flat index `start`.
+struct ChunkRows {
+    uint32_t start, ng, total;
+};
+
+__device__ __forceinline__ uint32_t lanemask_lt()
+{
+    uint32_t m;
+    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
+    return m;
+}
+
+__device__ __forceinline__ uint32_t lanemask_le()
+{
+    uint32_t m;
+    asm("mov.u32 %0, %%lanemask_le;" : "=r"(m));
+    return m;
+}
+
+__device__ __forceinline__ uint32_t warp_incl_scan(uint32_t x, uint32_t lane)
+{
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(kFull, x, o);
+        if (lane >= static_cast<uint32_t>(o)) x += t;
+    }
+    return x;
+}
+
+// Flattens the rows [beg, end) of the warp's lanes into 4-edge groups and writes the non-empty
+// ones, in lane order, to the stage.
+__device__ __forceinline__ ChunkRows publish_rows(WarpStage* st, int32_t beg, int32_t end, uint32_t lane)
+{
+    ChunkRows c;
+    c.ng = end > beg ? (static_cast<uint32_t>(end - 1) >> 2) - (static_cast<uint32_t>(beg) >> 2) + 1 : 0u;
+    const uint32_t incl = warp_incl_scan(c.ng, lane);
+    c.total = __shfl_sync(kFull, incl, 31);
+    c.start = incl - c.ng;
+    const uint32_t has = __ballot_sync(kFull, c.ng > 0);
+    if (c.ng > 0) {
+        const uint32_t r = __popc(has & lanemask_lt());
+        st->beg[r] = beg;
+        st->end[r] = end;
+        st->qoff[r] = (static_cast<uint32_t>(beg) >> 2) - c.start;
+        st->vert[r] = static_cast<uint8_t>(lane);
+    }
+    __syncwarp();
+    return c;
+}
+
+// The non-empty row that holds flat group t0 + lane. Every row that starts in the window
+// [t0, t0 + 32) sets the bit of its first group; a lane's owner is then the number of starts up to
+// its own bit. `owners` carries the rows that start before the window: call it for t0 = 0, 32, ...
+// in turn. One warp reduction and one population count take the place of a five-step shuffle
+// search and of the shuffles that fetched the row.
+__device__ __forceinline__ uint32_t window_owner(const ChunkRows& c, uint32_t t0, uint32_t& owners)
+{
+    const uint32_t d = c.start - t0;
+    const uint32_t starts = __reduce_or_sync(kFull, c.ng > 0 && d < 32 ? 1u << d : 0u);
+    const uint32_t r = owners + __popc(starts & lanemask_le()) - 1;
+    owners += __popc(starts);
+    return r;
+}
+
+// Appends the lane's live edges (flags ok0..ok3 of edges e0..e0+3, of row r) to the stage, which
+// holds `staged` <= 31; returns the new count.
+__device__ __forceinline__ uint32_t stage_live(WarpStage* st, uint32_t staged, bool ok0, bool ok1, bool ok2,
+                                               bool ok3, int32_t e0, uint32_t r, uint32_t lane)
+{
+    const uint32_t nc = (uint32_t)ok0 + (uint32_t)ok1 + (uint32_t)ok2 + (uint32_t)ok3;
+    const uint32_t incl = warp_incl_scan(nc, lane);
+    uint32_t p = staged + incl - nc;
+    if (ok0) { st->edge[p] = e0; st->src[p++] = static_cast<uint8_t>(r); }
+    if (ok1) { st->edge[p] = e0 + 1; st->src[p++] = static_cast<uint8_t>(r); }
+    if (ok2) { st->edge[p] = e0 + 2; st->src[p++] = static_cast<uint8_t>(r); }
+    if (ok3) { st->edge[p] = e0 + 3; st->src[p++] = static_cast<uint8_t>(r); }
+    staged += __shfl_sync(kFull, incl, 31);
+    __syncwarp();
+    return staged;
+}
+
 template <bool G>
 struct WarpSpace {
     uint32_t* lvl;
@@ -353,23 +446,6 @@ __device__ __forceinline__ uint32_t ld_shared_word(const uint32_t* p)
 struct SampleCounters {
     unsigned long long reached = 0, examined = 0, live = 0, nontree = 0, passes = 0, done = 0;
 };
-
-__device__ __forceinline__ uint32_t lanemask_lt()
-{
-    uint32_t m;
-    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
-    return m;
-}
-
-__device__ __forceinline__ uint32_t warp_incl_scan(uint32_t x, uint32_t lane)
-{
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(kFull, x, o);
-        if (lane >= static_cast<uint32_t>(o)) x += t;
-    }
-    return x;
-}
 
 __device__ __forceinline__ bool excluded(const uint32_t* excl, uint32_t v)
 {

@@ -106,17 +106,17 @@ cudaError_t launch_cta_tier(const SampleParams& P, const CtaCfg& c, uint32_t blo
 // Zero the per-slot visited bitmaps of a large-graph block tier (no-op for the shared variant).
 cudaError_t prepare_cta_scratch(const CtaCfg& c, uint32_t blocks, uint8_t* scratch, cudaStream_t s);
 
-// Monte-Carlo spread (spread.cu): adds sum over samples [0, P.theta) of |R| (seeds included) to
-// *sum, with the block tier's layout `c` and `blocks` slots of `scratch`.
-cudaError_t launch_spread(const SampleParams& P, const CtaCfg& c, uint32_t blocks, uint64_t smem,
-                          uint8_t* scratch, unsigned long long* sum, cudaStream_t s);
-
-// Spread of many blocker sets (spread.cu): for item i < items, adds |R| of sample i % P.theta with
-// set i / P.theta (k vertices of `sets`) blocked on top of P.excl into sums[i / P.theta].
-// *cursor must start at 0.
-cudaError_t launch_spread_sets(const SampleParams& P, const CtaCfg& c, uint32_t blocks, uint64_t smem,
-                               uint8_t* scratch, const int32_t* sets, uint32_t k, unsigned long long items,
-                               unsigned long long* cursor, unsigned long long* sums, cudaStream_t s);
+// Monte-Carlo spread (spread.cu) over items of (blocker set, sample): item i adds |R| (seeds
+// included) of sample i % P.theta, with set i / P.theta (k vertices of `sets`) blocked on top of
+// P.excl, to sums[i / P.theta]. A call enqueues slices 0 .. spread_slices(items) - 1 in order, with
+// the block tier's layout `c` and `blocks` slots of `scratch` and with spread_handoff_words(items)
+// words of `handoff` (shared by the slices). P.ctl->error must start at 0.
+unsigned long long spread_slices(unsigned long long items);
+uint64_t spread_handoff_words(unsigned long long items);
+cudaError_t launch_spread_slice(const SampleParams& P, const CtaCfg& c, uint32_t blocks, uint64_t smem,
+                                uint8_t* scratch, const int32_t* sets, uint32_t k, unsigned long long items,
+                                unsigned long long slice, uint32_t* handoff, unsigned long long* sums,
+                                cudaStream_t s);
 
 // Batched multi-query steps (batch.cu).
 bool plan_batch_cta(const DeviceInfo& dev, int32_t max_n, int32_t max_m, CtaCfg* c, uint32_t* blocks,
