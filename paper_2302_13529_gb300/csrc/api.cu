@@ -304,8 +304,8 @@ int setup_query(const imin_graph* g, const std::vector<int32_t>& seeds, uint32_t
     IMIN_CUDA(cudaMemsetAsync(q.excl, 0, sizeof(uint32_t) * q.words, s));
     IMIN_CUDA(cudaMemsetAsync(q.delta, 0, sizeof(unsigned long long) * g->n, s));
     IMIN_CUDA(cudaMemsetAsync(q.stats, 0, sizeof(unsigned long long) * kStCount, s));
-    IMIN_CUDA(cudaMemsetAsync(q.scratch1, 0xFF, q.plan.scratch_bytes[1], s));
-    IMIN_CUDA(cudaMemsetAsync(q.scratch2, 0xFF, q.plan.scratch_bytes[2], s));
+    IMIN_CUDA(prepare_warp_slots(q.plan, 1, q.scratch1, s));
+    IMIN_CUDA(prepare_warp_slots(q.plan, kTierWhole, q.scratch2, s));
     IMIN_CUDA(launch_build_excl(q.excl, q.seeds, static_cast<int32_t>(seeds.size()), s));
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return IMIN_OK;
@@ -1088,7 +1088,7 @@ int batch_impl(Driver which, imin_query* qs, int32_t nq, void* stream, uint32_t 
     if (global_bytes > 0)
         IMIN_CUDA(prepare_cta_scratch(cfg[kBatchGlobalClass], cta_blocks[kBatchGlobalClass], global_scratch, s));
     IMIN_CUDA(arena.alloc(&whole_scratch, wp.scratch_bytes[kTierWhole]));
-    IMIN_CUDA(cudaMemsetAsync(whole_scratch, 0xFF, wp.scratch_bytes[kTierWhole], s));
+    IMIN_CUDA(prepare_warp_slots(wp, kTierWhole, whole_scratch, s));
     IMIN_CUDA(arena.alloc(&stats, kStCount));
     // hand-off snapshots of the samples the warp tier gives up on, per size class after the
     // overflow items (at most 1 GiB in all; samples beyond the lists' room run from the start)

@@ -314,6 +314,7 @@ __global__ void __launch_bounds__(kWholeWarps * 32) k_batch_whole(BatchStep B, T
         item = __shfl_sync(kFull, item, 0);
         if (item >= count) break;
         const uint2 qj = B.over[item];
+        ready_slot(slot_ready(T.gscratch, T.warp_bytes, gridDim.x * kWholeWarps, gw), w.hkey, w.hcap, lane);
         const SampleParams P = params_of(B.q[qj.x], B.step - B.q[qj.x].start);
         const int rc = run_sample<true, false>(P, w, qj.y, lane, sc);
         if (lane == 0 && rc != kSampleDone)

@@ -403,6 +403,17 @@ __device__ __forceinline__ uint32_t stage_live(WarpStage* st, uint32_t staged, b
     return staged;
 }
 
+// The slots of tiers 1-2: one of warp_bytes per warp, then a `ready` word per warp (ready_slot).
+__host__ __device__ inline uint64_t slots_bytes(uint64_t warp_bytes, uint32_t warps)
+{
+    return warps * (warp_bytes + sizeof(uint32_t));
+}
+
+__host__ __device__ inline uint32_t* slot_ready(uint8_t* slots, uint64_t warp_bytes, uint32_t warps, uint64_t warp)
+{
+    return reinterpret_cast<uint32_t*>(slots + warp_bytes * warps) + warp;
+}
+
 template <bool G>
 struct WarpSpace {
     uint32_t* lvl;
@@ -450,6 +461,21 @@ struct SampleCounters {
 __device__ __forceinline__ bool excluded(const uint32_t* excl, uint32_t v)
 {
     return (__ldg(excl + (v >> 5)) >> (v & 31)) & 1u;
+}
+
+// Tiers 1-2 keep their hash empty between samples, but their slots start as they were allocated: a
+// whole-graph slot is so large (up to 1 GiB over all warps) that emptying every slot up front cost
+// a small call more than its samples did, while few calls ever reach these tiers. So a warp empties
+// its slot's hash when it takes the first sample on it; `ready`, zeroed with the allocation, says
+// that this was done.
+__device__ __forceinline__ void ready_slot(uint32_t* ready, uint32_t* hkey, uint32_t hcap, uint32_t lane)
+{
+    if (*ready != 0) return;
+    for (uint32_t i = lane; i < hcap / 4; i += 32)
+        reinterpret_cast<uint4*>(hkey)[i] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+    __syncwarp();
+    if (lane == 0) *ready = 1;
+    __syncwarp();
 }
 
 enum SampleResult { kSampleDone = 0, kSampleOverflow = 1, kSampleError = 2 };

@@ -89,11 +89,14 @@ TierPlan plan_tiers(const DeviceInfo& dev, int32_t n, int32_t m, uint32_t ns, ui
 
 // Enqueue tier `tier` of one Alg. 2 call (tier 0 takes samples [0, theta); tiers 1 and 2 take
 // the samples the previous tier could not hold). P.ctl must be zeroed and P.delta cleared
-// before tier 0; `scratch` must point at plan.scratch_bytes[tier] bytes whose hash words are
-// all 0xFF (tiers 1-2). Returns cudaSuccess without launching when the tier has no blocks.
+// before tier 0; `scratch` must point at plan.scratch_bytes[tier] bytes, prepared by
+// prepare_warp_slots (tiers 1-2). Returns cudaSuccess without launching when the tier has no blocks.
 // *launched is set to whether a kernel was enqueued.
 cudaError_t launch_sample_tier(int tier, const SampleParams& P, const TierPlan& plan,
                                uint8_t* scratch, cudaStream_t s, bool* launched);
+
+// Marks the freshly allocated slots of warp tier 1 or 2 as not yet emptied.
+cudaError_t prepare_warp_slots(const TierPlan& plan, int tier, uint8_t* scratch, cudaStream_t s);
 
 // Block-per-sample tier: layout, grid and shared memory. Graphs with n <= kCtaMaxVertices keep
 // the visited bitmap in shared memory; larger ones keep it in each block's global slot.

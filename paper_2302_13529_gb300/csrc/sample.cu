@@ -90,6 +90,7 @@ k_sample_tier(SampleParams P, TierCfg T)
             from_range ? P.theta : *reinterpret_cast<const volatile uint32_t*>(&P.ctl->count[kTier]);
         if (item >= total) break;
         const uint32_t j = from_range ? item : P.lists[kTier * P.theta + item];
+        if constexpr (G) ready_slot(slot_ready(T.gscratch, T.warp_bytes, gridDim.x * kWarpsPerBlock, gw), w.hkey, w.hcap, lane);
         uint32_t at[4];
         const int rc = run_sample<G, kClearAll, M>(P, w, j, lane, sc, at);
         if (rc == kSampleOverflow) {
@@ -231,7 +232,7 @@ TierPlan plan_tiers(const DeviceInfo& dev, int32_t n, int32_t m, uint32_t ns, ui
         p.warps_per_block[1] = kWarpsPerBlock;
         p.blocks[1] = p.use_cta ? 0u : b1 * dev.sms;
         p.smem_bytes[1] = kWarpsPerBlock * kStageBytes;
-        p.scratch_bytes[1] = c.warp_bytes * p.blocks[1] * kWarpsPerBlock;
+        p.scratch_bytes[1] = slots_bytes(c.warp_bytes, p.blocks[1] * kWarpsPerBlock);
     }
     // tier 2: per-warp global slot for any cascade (|R| <= n)
     {
@@ -248,9 +249,16 @@ TierPlan plan_tiers(const DeviceInfo& dev, int32_t n, int32_t m, uint32_t ns, ui
         p.warps_per_block[2] = kWarpsPerBlock;
         p.blocks[2] = blocks;
         p.smem_bytes[2] = kWarpsPerBlock * kStageBytes;
-        p.scratch_bytes[2] = c.warp_bytes * blocks * kWarpsPerBlock;
+        p.scratch_bytes[2] = slots_bytes(c.warp_bytes, blocks * kWarpsPerBlock);
     }
     return p;
+}
+
+cudaError_t prepare_warp_slots(const TierPlan& p, int tier, uint8_t* scratch, cudaStream_t s)
+{
+    const uint32_t warps = p.blocks[tier] * kWarpsPerBlock;
+    if (warps == 0) return cudaSuccess;
+    return cudaMemsetAsync(slot_ready(scratch, p.cfg[tier].warp_bytes, warps, 0), 0, sizeof(uint32_t) * warps, s);
 }
 
 cudaError_t launch_sample_tier(int tier, const SampleParams& P, const TierPlan& plan,

@@ -236,7 +236,7 @@ int imin_server::grow_plans(const std::vector<Req*>& active)
         if (whole_scratch) cudaFreeAsync(whole_scratch, s);
         const uint64_t bytes = whole.scratch_bytes[kTierWhole];
         if (cudaMallocAsync(&whole_scratch, bytes, s) != cudaSuccess) return IMIN_ERR_NOMEM;
-        if (cudaMemsetAsync(whole_scratch, 0xFF, bytes, s) != cudaSuccess) return IMIN_ERR_CUDA;
+        if (prepare_warp_slots(whole, kTierWhole, whole_scratch, s) != cudaSuccess) return IMIN_ERR_CUDA;
     }
     return IMIN_OK;
 }
