@@ -205,7 +205,6 @@ __host__ __device__ inline Handoff handoff_layout(uint32_t rcap, uint32_t dcap, 
 struct CtaCfg {
     uint32_t bm_words;    // visited bitmap words (>= n/32)
     uint32_t res_slots;   // resolution hash slots (power of two)
-    uint32_t res_shift;   // 32 - log2(res_slots)
     uint32_t rcap;        // local ids per slot
     uint32_t ecap;        // non-tree edges per slot
     uint32_t global_bitmap;  // 1: the bitmap is in the slot (large n); 0: in shared memory,

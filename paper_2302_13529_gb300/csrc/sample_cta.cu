@@ -128,9 +128,6 @@ bool plan_cta_tier(const DeviceInfo& dev, int32_t n, int32_t m, CtaCfg* c, uint3
     c->out_tier = kTierWhole;
     c->tree_words = smem_bitmap ? c->bm_words : 2 * slots;
     c->res_slots = slots;
-    uint32_t bits = 0;
-    while ((1u << bits) < slots) ++bits;
-    c->res_shift = 32 - bits;
     // every reached vertex fits when the bitmap is shared; large graphs cap the slot arrays and
     // hand bigger cascades to the whole-graph tier
     c->rcap = smem_bitmap ? static_cast<uint32_t>(n) + 1

@@ -20,9 +20,9 @@
 //   * per-vertex arrays indexed by local id (BFS discovery order) -- global id, BFS parent,
 //     immediate dominator -- live in a per-block slot of global memory that is written once
 //     per discovery and read back densely, so it streams through L2;
-//   * live edges to already-visited vertices ("non-tree" edges) are rare; their targets are
-//     resolved from global to local ids afterwards through a small hash built in the (then
-//     cleared) bitmap space, in chunks when there are many;
+//   * live edges to already-visited vertices ("non-tree" edges) are rare on most graphs; their
+//     targets are resolved from global to local ids afterwards, a few through a small hash built
+//     in the (then cleared) bitmap space, many through an array by global id in the slot;
 //   * dominators, subtree sizes and the counter update follow the same scheme as the warp
 //     tiers (imin_dev.cuh): iterated NCA folding over non-tree edges plus each target's BFS
 //     parent, a deepest-level-first subtree sweep, and 64-bit atomics into Delta.
@@ -224,8 +224,9 @@ __device__ __forceinline__ bool finish_tree(const SampleParams& P, CtaShared<T>&
 }
 
 // The dominator passes of finish_tree on packed shared-memory words, one per local id,
-// (idom << 16) | c with c = 0 (every id fits: nR <= K), so atomicMin on the word is atomicMin on
-// idom.
+// (idom << 16) | c with c = 1 (every id fits: nR <= K), so atomicMin on the word is atomicMin on
+// idom. One warp alone for the few non-tree edges of most samples, with a vote in place of the two
+// barriers, was no faster.
 template <uint32_t T>
 __device__ __forceinline__ bool tree_passes_packed(const Slot& S, uint32_t* w, uint32_t nR, uint32_t nE,
                                                    uint32_t tid, uint32_t* passes_out)
@@ -234,25 +235,28 @@ __device__ __forceinline__ bool tree_passes_packed(const Slot& S, uint32_t* w, u
     volatile uint32_t* vw = w;
     bool broken = false;
     uint32_t passes = 0;
+    // one edge: idom(e.y) falls to the nearest common ancestor of itself, e.x and the parent
+    auto fold = [&](const uint2& e, uint32_t parent) -> bool {
+        uint32_t a = vw[e.y] >> 16, b = e.x;
+        for (uint32_t g = 0; a != b; ++g) {
+            if (g > 2 * nR) { broken = true; a = 0; break; }
+            nca_step(a, b, [&](uint32_t x) { return vw[x] >> 16; });
+        }
+        b = parent;
+        for (uint32_t g = 0; a != b; ++g) {
+            if (g > 2 * nR) { broken = true; a = 0; break; }
+            nca_step(a, b, [&](uint32_t x) { return vw[x] >> 16; });
+        }
+        if (broken || a >= (vw[e.y] >> 16)) return false;
+        const uint32_t lowered = (a << 16) | 1u;
+        return lowered < atomicMin(w + e.y, lowered);
+    };
     if (nE > 0) {
         for (;;) {
             int changed = 0;
             for (uint32_t k = tid; k < nE; k += kCtaThreads) {
                 const uint2 e = S.edges[k];
-                uint32_t a = vw[e.y] >> 16, b = e.x;
-                for (uint32_t g = 0; a != b; ++g) {
-                    if (g > 2 * nR) { broken = true; a = 0; break; }
-                    nca_step(a, b, [&](uint32_t x) { return vw[x] >> 16; });
-                }
-                b = S.par[e.y];
-                for (uint32_t g = 0; a != b; ++g) {
-                    if (g > 2 * nR) { broken = true; a = 0; break; }
-                    nca_step(a, b, [&](uint32_t x) { return vw[x] >> 16; });
-                }
-                if (!broken && a < (vw[e.y] >> 16)) {
-                    const uint32_t old = atomicMin(w + e.y, a << 16);
-                    changed |= (a << 16) < old;
-                }
+                changed |= fold(e, S.par[e.y]);
             }
             ++passes;
             broken = __syncthreads_or(broken);
@@ -354,7 +358,8 @@ __device__ __forceinline__ bool tree_passes16(CtaShared<T>& sh, const Slot& S, u
 // dominators are final, with the first K local ids -- the shallowest BFS levels -- as packed
 // shared-memory words (idom << 16) | c and ids K..nR-1 (kSplit) on the slot arrays (idom in
 // S.idom; c in S.par, which is dead once the passes end). For trees of fewer than 2^16
-// vertices: c < 2^16 never carries into idom. On entry w[i] = idom(i) << 16 for i < K.
+// vertices: c < 2^16 never carries into idom. On entry w[i] = (idom(i) << 16) | 1 for i < K; on
+// return it is 0.
 template <bool kSplit, uint32_t T>
 __device__ __forceinline__ void tree_sweep_packed(const SampleParams& P, CtaShared<T>& sh, const Slot& S,
                                                   uint32_t* w, uint32_t K, uint32_t nR, uint32_t nlev,
@@ -370,11 +375,12 @@ __device__ __forceinline__ void tree_sweep_packed(const SampleParams& P, CtaShar
         if (!kSplit || x < K) return vw[x] & 0xFFFFu;
         return __ldcg(S.par + x);
     };
-    for (uint32_t i = tid; i < K; i += kCtaThreads) w[i] = (vw[i] & 0xFFFF0000u) | 1u;
     if constexpr (kSplit) {
         for (uint32_t i = K + tid; i < nR; i += kCtaThreads) S.par[i] = 1;
     }
     __syncthreads();
+    // (runs of small levels left to one warp, without the barriers between them: 2 % slower on the
+    // mid workload, where one warp's chain is longer than the barriers it saves)
     for (uint32_t d = nlev - 1; d >= 1; --d) {
         const uint32_t b0 = sh.lvl[d], b1 = sh.lvl[d + 1];
         for (uint32_t i = b0 + tid; i < b1; i += kCtaThreads) {
@@ -384,8 +390,10 @@ __device__ __forceinline__ void tree_sweep_packed(const SampleParams& P, CtaShar
         }
         __syncthreads();
     }
-    for (uint32_t i = 1 + ns + tid; i < nR; i += kCtaThreads)
-        atomicAdd(P.delta + S.gid[i], static_cast<unsigned long long>(c_of(i)));
+    for (uint32_t i = tid; i < nR; i += kCtaThreads) {
+        if (i > ns) atomicAdd(P.delta + S.gid[i], static_cast<unsigned long long>(c_of(i)));
+        if (!kSplit || i < K) w[i] = 0;
+    }
     __syncthreads();
 }
 
@@ -447,7 +455,9 @@ __device__ __forceinline__ int run_sample_cta(const SampleParams& P, const CtaCf
 {
     constexpr uint32_t kCtaThreads = T, kCtaWarps = CtaDims<T>::kWarps, kChunk = CtaDims<T>::kChunk;
     const uint32_t ns = P.ns;
-    const uint32_t lane = tid & 31, wid = tid >> 5;
+    // the warp's index through a shuffle, so that the compiler knows it to be the same in all lanes
+    // and keeps the group loop, whose bound depends on it, free of divergence handling
+    const uint32_t lane = tid & 31, wid = __shfl_sync(kFull, tid >> 5, 0);
     uint32_t lb = 1, le = 1 + ns, nlev = 1;
     if (from == nullptr) {
         for (uint32_t i = tid; i < ns; i += kCtaThreads) {
@@ -524,7 +534,8 @@ __device__ __forceinline__ int run_sample_cta(const SampleParams& P, const CtaCf
 
             // ---- groups: one per thread per iteration; live edges accumulate in the warp's
             // stage, which is visited by the full warp whenever it is at least half full and
-            // once more at the end of the chunk
+            // once more at the end of the chunk; a warp leaves the loop when its own groups end
+            // (mid workload, 50 rounds: 241.2 -> 237.6 ms in this kernel)
             uint32_t staged = 0;  // warp-uniform
             // the owner row and thresholds of the thread's next group are fetched while the
             // current group's Philox runs
@@ -557,7 +568,7 @@ __device__ __forceinline__ int run_sample_cta(const SampleParams& P, const CtaCf
                 }
             };
             fetch(tid);
-            for (uint32_t t0 = 0; t0 < total; t0 += kCtaThreads) {
+            for (uint32_t t0 = 0; t0 + wid * 32 < total; t0 += kCtaThreads) {
                 const uint32_t q = nq, ul = nul;
                 const int32_t ob = nob, oe = noe;
                 const uint4 th = nth;
@@ -620,33 +631,48 @@ __device__ __forceinline__ int run_sample_cta(const SampleParams& P, const CtaCf
         return kSampleDone;
     }
 
-    // non-tree edge targets: global id -> local id through a hash in the bitmap space, in
-    // chunks of at most half the hash's slots
-    if (nE > 0) {
+    // non-tree edge targets: global id -> local id. Few edges: through a hash in the bitmap space
+    // sized to them, so that emptying it costs no more than they do. More than half the hash's
+    // slots: through an array by global id in the rows' space, which the BFS no longer needs and
+    // which holds n words unless the slots are capped below n vertices; it needs no emptying,
+    // because every target was reached, so its entry is written before it is read. Trivalency on
+    // R-MAT 2^17 (12,491 vertices and 15,646 non-tree edges per sample) took 16 passes of the hash,
+    // each over all vertices, 37 % of the block's time; GreedyReplace there: 162 -> 118 ms.
+    if (nE > C.res_slots / 2 && C.rcap > static_cast<uint32_t>(P.g.n)) {
+        uint32_t* local = reinterpret_cast<uint32_t*>(S.rows);
+        for (uint32_t i = 1 + ns + tid; i < nR; i += kCtaThreads) __stcg(local + S.gid[i], i);
+        __syncthreads();
+        for (uint32_t k = tid; k < nE; k += kCtaThreads) S.edges[k].y = __ldcg(local + S.edges[k].y);
+        __syncthreads();
+    } else if (nE > 0) {
         uint32_t* keys = res;
-        uint32_t* vals = res + C.res_slots;
-        const uint32_t hmask = C.res_slots - 1;
-        for (uint32_t c0 = 0; c0 < nE; c0 += C.res_slots / 2) {
-            const uint32_t c1 = min(nE, c0 + C.res_slots / 2);
-            for (uint32_t i = tid; i < C.res_slots; i += kCtaThreads) keys[i] = kEmpty;
+        const uint32_t most = C.res_slots / 2;
+        uint32_t h = 64;
+        while (h < 2 * min(nE, most)) h <<= 1;
+        h = min(h, C.res_slots);
+        uint32_t* vals = res + h;
+        const uint32_t hmask = h - 1, hshift = __clz(h) + 1;
+        for (uint32_t c0 = 0; c0 < nE; c0 += most) {
+            const uint32_t c1 = min(nE, c0 + most);
+            for (uint32_t i = tid; i < h; i += kCtaThreads) keys[i] = kEmpty;
             __syncthreads();
             for (uint32_t k = c0 + tid; k < c1; k += kCtaThreads)
-                res_slot(keys, hmask, C.res_shift, S.edges[k].y, true);
+                res_slot(keys, hmask, hshift, S.edges[k].y, true);
             __syncthreads();
             for (uint32_t i = 1 + ns + tid; i < nR; i += kCtaThreads) {
-                const uint32_t s = res_slot(keys, hmask, C.res_shift, static_cast<uint32_t>(S.gid[i]), false);
+                const uint32_t s = res_slot(keys, hmask, hshift, static_cast<uint32_t>(S.gid[i]), false);
                 if (s != kEmpty) vals[s] = i;
             }
             __syncthreads();
             for (uint32_t k = c0 + tid; k < c1; k += kCtaThreads) {
-                const uint32_t s = res_slot(keys, hmask, C.res_shift, S.edges[k].y, false);
+                const uint32_t s = res_slot(keys, hmask, hshift, S.edges[k].y, false);
                 if (s == kEmpty) broken = true;  // every target was reached: cannot happen
                 else S.edges[k].y = vals[s];
             }
             __syncthreads();
         }
         if constexpr (kResInBitmap) {
-            for (uint32_t i = tid; i < 2 * C.res_slots; i += kCtaThreads) bm[i] = 0;
+            for (uint32_t i = tid; i < 2 * h; i += kCtaThreads) bm[i] = 0;
         }
         broken = __syncthreads_or(broken);
         if (broken) return kSampleError;
@@ -661,20 +687,16 @@ __device__ __forceinline__ int run_sample_cta(const SampleParams& P, const CtaCf
     if (nR < (1u << 16)) {
         const uint32_t K = min(nR, C.tree_words);
         if (K == nR) {
-            for (uint32_t i = tid; i < K; i += kCtaThreads) res[i] = S.idom[i] << 16;
+            for (uint32_t i = tid; i < K; i += kCtaThreads) res[i] = (S.idom[i] << 16) | 1u;
             __syncthreads();
             broken = tree_passes_packed<T>(S, res, nR, nE, tid, &passes);
             tree_sweep_packed<false>(P, sh, S, res, K, nR, nlev, ns, tid);
         } else {
             broken = tree_passes16(sh, S, reinterpret_cast<uint16_t*>(res), 2 * C.tree_words, nR, nE, tid,
                                    &passes);
-            for (uint32_t i = tid; i < K; i += kCtaThreads) res[i] = ld_tree(S.idom + i) << 16;
+            for (uint32_t i = tid; i < K; i += kCtaThreads) res[i] = (ld_tree(S.idom + i) << 16) | 1u;
             __syncthreads();
             tree_sweep_packed<true>(P, sh, S, res, K, nR, nlev, ns, tid);
-        }
-        if constexpr (kResInBitmap) {
-            for (uint32_t i = tid; i < K; i += kCtaThreads) res[i] = 0;  // it is the bitmap
-            __syncthreads();
         }
     } else {
         broken = finish_tree(P, sh, S, S.idom, S.par, nR, nE, nlev, ns, tid, &passes);
