@@ -22,7 +22,7 @@ using namespace sel;
 
 constexpr uint32_t kWholeWarps = 8;  // warps per block of the batched whole-graph kernel
 constexpr uint32_t kBatchWarps = 8;  // warps per block of the batched warp-tier kernel
-constexpr uint64_t kWarpStageBytes = kStageCap * sizeof(uint2);
+constexpr uint64_t kWarpStageBytes = sizeof(WarpStage);
 
 // Largest q with prefix[q] <= item (prefix[0] = 0, item < prefix[nq]).
 __device__ __forceinline__ uint32_t find_query(const unsigned long long* prefix, uint32_t nq,
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 4) k_batch_warp(BatchStep B,
     uint8_t* base = mine + kWarpStageBytes;
     const WarpLayout L = warp_layout(T.rcap, T.hcap, T.ecap, T.dcap, false);
     WarpSpace<false> w;
-    w.stage = reinterpret_cast<uint2*>(mine);
+    w.stage = reinterpret_cast<WarpStage*>(mine);
     w.lvl = reinterpret_cast<uint32_t*>(base + L.lvl);
     w.hkey = reinterpret_cast<uint32_t*>(base + L.hkey);
     w.hval = reinterpret_cast<uint32_t*>(base + L.hval);
@@ -285,13 +285,13 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 4) k_batch_warp(BatchStep B,
 // The samples the block tier handed over, one warp each, with whole-graph capacity.
 __global__ void __launch_bounds__(kWholeWarps * 32) k_batch_whole(BatchStep B, TierCfg T)
 {
-    __shared__ __align__(16) uint2 stage[kWholeWarps][kStageCap];
+    __shared__ WarpStage stage[kWholeWarps];
     const uint32_t lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const uint64_t gw = static_cast<uint64_t>(blockIdx.x) * kWholeWarps + wib;
     uint8_t* base = T.gscratch + gw * T.warp_bytes;
     const WarpLayout L = warp_layout(T.rcap, T.hcap, T.ecap, T.dcap, true);
     WarpSpace<true> w;
-    w.stage = stage[wib];
+    w.stage = &stage[wib];
     w.lvl = reinterpret_cast<uint32_t*>(base + L.lvl);
     w.hkey = reinterpret_cast<uint32_t*>(base + L.hkey);
     w.hval = reinterpret_cast<uint32_t*>(base + L.hval);

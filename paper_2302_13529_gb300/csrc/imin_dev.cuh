@@ -6,8 +6,12 @@
 //   1. a level-synchronous BFS from the seeds (all at depth 0 under a virtual super-seed,
 //      Sec. 4 "From Multiple Seeds to One Seed"). The out-edges of a frontier are flattened
 //      into groups of 4 consecutive edge ids; each lane takes one group, loads its 4
-//      thresholds with one 16-byte load, evaluates one Philox4x32-10 call whose 4 output words
-//      decide the 4 edges, and loads the target id only for live edges. Live targets that are
+//      thresholds with one 16-byte load and evaluates one Philox4x32-10 call whose 4 output words
+//      decide the 4 edges. The ids of live edges wait in shared memory until 32 of them (or the
+//      chunk's last) can be visited with a lane each: the target is loaded only then. This kernel
+//      is bound by instruction issue, and with a few percent of the edges live, visiting them as
+//      they came left most lanes idle: 48 queries of the trivalency batch 36.3 -> 29.0 ms in the
+//      warp tier, the mid workload 33.2 -> 32.5 ms. Targets that are
 //      neither seeds nor blocked go through a warp-shared open-addressing hash (global id ->
 //      local id). A newly inserted vertex gets the next local id, so local ids follow BFS
 //      discovery order and every level occupies a contiguous id range; the discovering vertex
@@ -48,7 +52,6 @@ constexpr int kTiers = 4;
 constexpr int kTierWhole = 2;
 constexpr int kTierCta = 3;
 constexpr int32_t kCtaMaxVertices = 1 << 18;
-constexpr int kStageCap = 128;  // 32 lanes x 4 edges per group
 
 enum : uint32_t { kErrCapacity = 1u, kErrInternal = 2u };
 
@@ -312,13 +315,13 @@ __host__ __device__ inline WarpLayout warp_layout(uint32_t rcap, uint32_t hcap, 
 // Shared-memory work area of one warp's frontier chunk (always shared memory).
 // The non-empty rows of up to 32 frontier vertices, in order, and the live edges that wait to be
 // visited: at most 31 left over plus one iteration's 32 lanes x 4 edges.
-constexpr uint32_t kLiveCap = 160;
+constexpr uint32_t kStageCap = 160;
 struct __align__(16) WarpStage {
-    uint32_t edge[kLiveCap];  // live edge ids
+    uint32_t edge[kStageCap];  // live edge ids
     int32_t beg[32], end[32];  // edge range of each non-empty row
     uint32_t qoff[32];         // the row's 4-edge group of flat index t is qoff + t
     uint8_t vert[32];          // the row's vertex: its position in the chunk
-    uint8_t src[kLiveCap];    // the staged edge's row
+    uint8_t src[kStageCap];    // the staged edge's row
 };
 
 // The flattened 4-edge groups of a chunk: a lane's own row starts at flat index `start`.
@@ -423,7 +426,7 @@ struct WarpSpace {
     uint32_t* par;   // BFS parent (idom before the dominator passes)
     uint32_t* hslot;
     uint2* edges;
-    uint2* stage;  // always shared memory, kStageCap entries
+    WarpStage* stage;  // always shared memory
     uint32_t rcap, hcap, hbits, ecap, dcap;
 };
 
@@ -506,7 +509,7 @@ __device__ __forceinline__ int run_sample(const SampleParams& P, const WarpSpace
     uint32_t nE = 0;       // non-tree edges
     uint32_t nlev = 1;     // completed levels; level d = [lvl[d], lvl[d+1])
     bool over = false;
-    unsigned long long examined = 0, live = 0;
+    uint32_t examined = 0, live = 0;  // per lane: at most m
 
     uint32_t lb = 1, le = 1 + ns;
     uint32_t nE_level = 0;  // non-tree edges recorded before the current level
@@ -522,41 +525,26 @@ __device__ __forceinline__ int run_sample(const SampleParams& P, const WarpSpace
                 end = __ldg(P.g.row_ptr + u + 1);
             }
             examined += static_cast<uint32_t>(end - beg);
-            const uint32_t ng =
-                end > beg ? (static_cast<uint32_t>(end - 1) >> 2) - (static_cast<uint32_t>(beg) >> 2) + 1
-                          : 0u;
-            const uint32_t incl = warp_incl_scan(ng, lane);
-            const uint32_t total = __shfl_sync(kFull, incl, 31);
-
-            for (uint32_t t0 = 0; t0 < total && !over; t0 += 32) {
-                const uint32_t t = t0 + lane;
-                // owner lane: the first lane whose inclusive group count exceeds t
-                uint32_t pos = 0;
-#pragma unroll
-                for (uint32_t step = 16; step >= 1; step >>= 1) {
-                    const uint32_t v = __shfl_sync(kFull, incl, pos + step - 1);
-                    if (v <= t) pos += step;
-                }
-                const uint32_t o_incl = __shfl_sync(kFull, incl, pos);
-                const uint32_t o_ng = __shfl_sync(kFull, ng, pos);
-                const int32_t o_beg = __shfl_sync(kFull, beg, pos);
-                const int32_t o_end = __shfl_sync(kFull, end, pos);
-
+            const ChunkRows rows = publish_rows(w.stage, beg, end, lane);
+            uint32_t owners = 0;  // non-empty rows that start before the current window
+            uint32_t staged = 0;  // live edges waiting in the stage
+            for (uint32_t t0 = 0; t0 < rows.total && !over; t0 += 32) {
+                const uint32_t r = window_owner(rows, t0, owners);
                 bool ok0 = false, ok1 = false, ok2 = false, ok3 = false;
-                uint32_t v0 = 0, v1 = 0, v2 = 0, v3 = 0;
-                const uint32_t ul = base + pos;
-                if (t < total) {
-                    const uint32_t q = (static_cast<uint32_t>(o_beg) >> 2) + (t - (o_incl - o_ng));
+                int32_t e0 = 0;
+                if (t0 + lane < rows.total) {
+                    const int32_t o_beg = w.stage->beg[r], o_end = w.stage->end[r];
+                    const uint32_t q = w.stage->qoff[r] + t0 + lane;
                     const uint4 th = __ldg(P.g.thr4 + q);
-                    const int32_t e0 = static_cast<int32_t>(q << 2);
+                    e0 = static_cast<int32_t>(q << 2);
                     // the IC decision of group_live written out as four flags (measured 2-5 %
                     // faster on the warp tiers than testing a materialised mask)
                     if (M == kModelIC || (M == kModelAny && P.g.lo4 == nullptr)) {
-                        const uint4 r = philox4x32_10(make_uint4(q, j, P.round, 0u), P.key_lo, P.key_hi);
-                        ok0 = (e0 + 0 >= o_beg) && (e0 + 0 < o_end) && (r.x <= th.x);
-                        ok1 = (e0 + 1 >= o_beg) && (e0 + 1 < o_end) && (r.y <= th.y);
-                        ok2 = (e0 + 2 >= o_beg) && (e0 + 2 < o_end) && (r.z <= th.z);
-                        ok3 = (e0 + 3 >= o_beg) && (e0 + 3 < o_end) && (r.w <= th.w);
+                        const uint4 x = philox4x32_10(make_uint4(q, j, P.round, 0u), P.key_lo, P.key_hi);
+                        ok0 = (e0 + 0 >= o_beg) && (e0 + 0 < o_end) && (x.x <= th.x);
+                        ok1 = (e0 + 1 >= o_beg) && (e0 + 1 < o_end) && (x.y <= th.y);
+                        ok2 = (e0 + 2 >= o_beg) && (e0 + 2 < o_end) && (x.z <= th.z);
+                        ok3 = (e0 + 3 >= o_beg) && (e0 + 3 < o_end) && (x.w <= th.w);
                     } else {
                         const uint32_t lm = group_live<M>(P.g, q, th, o_beg, o_end, j, P.round, P.key_lo, P.key_hi);
                         ok0 = (lm & 1u) != 0;
@@ -564,33 +552,24 @@ __device__ __forceinline__ int run_sample(const SampleParams& P, const WarpSpace
                         ok2 = (lm & 4u) != 0;
                         ok3 = (lm & 8u) != 0;
                     }
-                    if (ok0) { v0 = static_cast<uint32_t>(__ldg(P.g.col + e0 + 0)); ok0 = !excluded(P.excl, v0); }
-                    if (ok1) { v1 = static_cast<uint32_t>(__ldg(P.g.col + e0 + 1)); ok1 = !excluded(P.excl, v1); }
-                    if (ok2) { v2 = static_cast<uint32_t>(__ldg(P.g.col + e0 + 2)); ok2 = !excluded(P.excl, v2); }
-                    if (ok3) { v3 = static_cast<uint32_t>(__ldg(P.g.col + e0 + 3)); ok3 = !excluded(P.excl, v3); }
                 }
-                const uint32_t nc = (uint32_t)ok0 + (uint32_t)ok1 + (uint32_t)ok2 + (uint32_t)ok3;
-                live += nc;
-                const uint32_t cincl = warp_incl_scan(nc, lane);
-                const uint32_t ctot = __shfl_sync(kFull, cincl, 31);
-                if (ctot == 0) continue;
-                {
-                    uint32_t p = cincl - nc;
-                    if (ok0) w.stage[p++] = make_uint2(ul, v0);
-                    if (ok1) w.stage[p++] = make_uint2(ul, v1);
-                    if (ok2) w.stage[p++] = make_uint2(ul, v2);
-                    if (ok3) w.stage[p++] = make_uint2(ul, v3);
-                }
-                __syncwarp();
+                staged = stage_live(w.stage, staged, ok0, ok1, ok2, ok3, e0, r, lane);
+                const bool last = t0 + 32 >= rows.total;
 
-                // ---- insert the staged live targets, one per lane per step
-                for (uint32_t s0 = 0; s0 < ctot; s0 += 32) {
-                    const bool act = s0 + lane < ctot;
+                // ---- visit the staged live edges, one per lane per step: full warps while the
+                // chunk goes on, the rest at its end
+                while (staged >= 32 || (last && staged > 0)) {
+                    const uint32_t take = staged < 32 ? staged : 32;
+                    staged -= take;
+                    bool act = lane < take;
                     uint32_t st = 0, slot = 0, cu = 0, cv = 0;
                     if (act) {
-                        const uint2 c = w.stage[s0 + lane];
-                        cu = c.x;
-                        cv = c.y;
+                        cu = base + w.stage->vert[w.stage->src[staged + lane]];
+                        cv = static_cast<uint32_t>(__ldg(P.g.col + w.stage->edge[staged + lane]));
+                        act = !excluded(P.excl, cv);
+                        live += act;
+                    }
+                    if (act) {
                         slot = (cv * 0x9E3779B1u) >> hshift;
                         for (uint32_t probe = 0; probe < w.hcap; ++probe) {
                             const uint32_t k = ld_shared_word<G>(w.hkey + slot);
@@ -630,7 +609,10 @@ __device__ __forceinline__ int run_sample(const SampleParams& P, const WarpSpace
                     const uint32_t epos = nE + __popc(ntm & lanemask_lt());
                     if (nt && epos < w.ecap) w.edges[epos] = make_uint2(cu, vl);
                     nE += __popc(ntm);
-                    if (__any_sync(kFull, bad) || nE > w.ecap || nR > w.rcap) over = true;
+                    if (__any_sync(kFull, bad) || nE > w.ecap || nR > w.rcap) {
+                        over = true;
+                        break;
+                    }
                 }
                 __syncwarp();
             }

@@ -18,7 +18,7 @@ namespace imin {
 namespace {
 
 constexpr uint32_t kWarpsPerBlock = 8;
-constexpr uint32_t kStageBytes = kStageCap * sizeof(uint2);
+constexpr uint32_t kStageBytes = sizeof(WarpStage);
 
 uint32_t next_pow2(uint64_t x)
 {
@@ -41,8 +41,15 @@ uint32_t env_u32(const char* name, uint32_t dflt)
     return static_cast<uint32_t>(std::strtoul(v, nullptr, 10));
 }
 
-template <int kTier, int M>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
+// Tier 0 comes in two register budgets. kPerSm = 5 blocks per SM (48 registers, a few spilled) is
+// for many samples: 2*10^4 linear-threshold samples of the mid graph 1.44 ms against 1.59 with 4.
+// With at most kFewPerWarp samples per warp, the call ends when each warp's one or two samples do,
+// so latency counts and not warps per SM, and kPerSm = 4 (64 registers) is faster: 10 rounds of
+// 10^4 samples on a 2,000-vertex graph 0.64 ms against 0.73.
+constexpr uint32_t kManyPerSm = 5, kFewPerSm = 4, kFewPerWarp = 2;
+
+template <int kTier, int M, uint32_t kPerSm = 1>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, kPerSm)
 k_sample_tier(SampleParams P, TierCfg T)
 {
     constexpr bool G = kTier > 0;
@@ -60,7 +67,7 @@ k_sample_tier(SampleParams P, TierCfg T)
     const WarpLayout L = warp_layout(T.rcap, T.hcap, T.ecap, T.dcap, !kClearAll);
 
     WarpSpace<G> w;
-    w.stage = reinterpret_cast<uint2*>(my_smem);
+    w.stage = reinterpret_cast<WarpStage*>(my_smem);
     w.lvl = reinterpret_cast<uint32_t*>(base + L.lvl);
     w.hkey = reinterpret_cast<uint32_t*>(base + L.hkey);
     w.hval = reinterpret_cast<uint32_t*>(base + L.hval);
@@ -165,8 +172,10 @@ void tier0_cfg(uint32_t ns, uint32_t r0, TierCfg* c)
 
 void allow_tier0_smem(const DeviceInfo& dev)
 {
-    allow_max_dynamic_smem(k_sample_tier<0, kModelLT>, dev);
-    allow_max_dynamic_smem(k_sample_tier<0, kModelIC>, dev);
+    allow_max_dynamic_smem(k_sample_tier<0, kModelLT, kManyPerSm>, dev);
+    allow_max_dynamic_smem(k_sample_tier<0, kModelIC, kManyPerSm>, dev);
+    allow_max_dynamic_smem(k_sample_tier<0, kModelLT, kFewPerSm>, dev);
+    allow_max_dynamic_smem(k_sample_tier<0, kModelIC, kFewPerSm>, dev);
 }
 
 void plan_tier0(const DeviceInfo& dev, uint32_t ns, uint32_t cutoff, TierPlan* p)
@@ -175,9 +184,9 @@ void plan_tier0(const DeviceInfo& dev, uint32_t ns, uint32_t cutoff, TierPlan* p
     p->warps_per_block[0] = kWarpsPerBlock;
     p->smem_bytes[0] = kWarpsPerBlock * (kStageBytes + p->cfg[0].warp_bytes);
     p->scratch_bytes[0] = 0;
-    // 5 blocks of 48 registers a thread share an SM; blocks that do not fit at once find the work
+    // kManyPerSm blocks share an SM at small cutoffs; blocks that do not fit at once find the work
     // cursor where the resident ones left it
-    p->blocks[0] = p->smem_bytes[0] <= dev.smem_optin ? 5u * dev.sms : 0u;
+    p->blocks[0] = p->smem_bytes[0] <= dev.smem_optin ? kManyPerSm * dev.sms : 0u;
 }
 
 TierPlan plan_tiers(const DeviceInfo& dev, int32_t n, int32_t m, uint32_t ns, uint32_t cutoff)
@@ -211,7 +220,7 @@ TierPlan plan_tiers(const DeviceInfo& dev, int32_t n, int32_t m, uint32_t ns, ui
         int occ = 0;
         if (p.smem_bytes[0] <= dev.smem_optin) {
             allow_tier0_smem(dev);
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sample_tier<0, kModelIC>,
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sample_tier<0, kModelIC, kManyPerSm>,
                                                           kWarpsPerBlock * 32, p.smem_bytes[0]);
         }
         p.blocks[0] = static_cast<uint32_t>(std::max(occ, 0)) * dev.sms;
@@ -275,14 +284,17 @@ cudaError_t launch_sample_tier(int tier, const SampleParams& P, const TierPlan& 
     // the first tier that runs takes the whole sample range; tier 0 is skipped only when the
     // seed set does not fit its shared-memory working set
     c.from_range = tier == 0 || (tier == 1 && plan.blocks[0] == 0 && !plan.use_cta);
+    const bool few = tier == 0 && P.theta <= kFewPerWarp * kWarpsPerBlock * plan.blocks[0];
     const dim3 grid(plan.blocks[tier]), block(kWarpsPerBlock * 32);
     const size_t sm = plan.smem_bytes[tier];
     if (P.g.lo4 == nullptr) {
-        if (tier == 0) k_sample_tier<0, kModelIC><<<grid, block, sm, s>>>(P, c);
+        if (few) k_sample_tier<0, kModelIC, kFewPerSm><<<grid, block, sm, s>>>(P, c);
+        else if (tier == 0) k_sample_tier<0, kModelIC, kManyPerSm><<<grid, block, sm, s>>>(P, c);
         else if (tier == 1) k_sample_tier<1, kModelIC><<<grid, block, sm, s>>>(P, c);
         else k_sample_tier<2, kModelIC><<<grid, block, sm, s>>>(P, c);
     } else {
-        if (tier == 0) k_sample_tier<0, kModelLT><<<grid, block, sm, s>>>(P, c);
+        if (few) k_sample_tier<0, kModelLT, kFewPerSm><<<grid, block, sm, s>>>(P, c);
+        else if (tier == 0) k_sample_tier<0, kModelLT, kManyPerSm><<<grid, block, sm, s>>>(P, c);
         else if (tier == 1) k_sample_tier<1, kModelLT><<<grid, block, sm, s>>>(P, c);
         else k_sample_tier<2, kModelLT><<<grid, block, sm, s>>>(P, c);
     }

@@ -1,0 +1,95 @@
+"""The routes a sampled cascade can take through the kernels, at the sizes where they change:
+the warp spread kernel's queue and its hand-off, the non-tree target array of the block tier, and
+the three launches of the allocation-free call. Counters and sums are integers: tolerance 0."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2302_13529_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _graph(n, src, dst, p, lt=False):
+    """A graph from edge lists with one probability for all edges (LT: weights of 1 / in-degree)."""
+    order = np.lexsort((dst, src))
+    src, dst = np.asarray(src)[order], np.asarray(dst, np.int32)[order]
+    row = np.zeros(n + 1, np.int32)
+    row[1:] = np.cumsum(np.bincount(src, minlength=n))
+    w = W.lt_wc_weights(dst, n) if lt else np.full(len(dst), int(p * 2**32) - 1, np.uint32)
+    return W.Graph(n, row, dst, w)
+
+
+def _star(leaves, p=1.0, chain=1):
+    """Vertex 0 -> `leaves` vertices, then a chain after the last leaf (the queue fills in one level)."""
+    n = 1 + leaves + chain
+    src = [0] * leaves + list(range(leaves, leaves + chain))
+    dst = list(range(1, leaves + 1)) + list(range(leaves + 1, leaves + chain + 1))
+    return _graph(n, src, dst, p)
+
+
+@pytest.mark.parametrize("leaves", [1, 31, 32, 33, 254, 255, 256, 257, 300, 1000])
+@pytest.mark.parametrize("p", [1.0, 0.97])
+def test_spread_around_the_queue_size(cuda_lib, leaves, p):
+    g = _star(leaves, p)
+    gh = cuda_lib.load_graph(g)
+    for theta in (1, 7, 65):
+        assert cuda_lib.estimate_spread(gh, [0], [], theta, 9, 2) == O.spread(g, [0], [], theta, 9, 2)
+        st = cuda_lib.last_stats()
+        assert st["samples"] == theta and st["reached"] == O.spread(g, [0], [], theta, 9, 2)
+        if p == 1.0:  # every edge is live and examined once per sample, on either route
+            assert st["examined_edges"] == theta * g.m and st["live_edges"] == theta * g.m
+
+
+@pytest.mark.parametrize("model", ["ic", "lt"])
+@pytest.mark.parametrize("k", [1, 3, 64])
+def test_spread_sets_across_grabs_and_routes(cuda_lib, model, k):
+    rng = np.random.default_rng(k)
+    n, m = 900, 5000
+    e = np.unique(rng.integers(0, n * n, m))
+    e = e[e // n != e % n]
+    g = _graph(n, e // n, e % n, 0.3, lt=model == "lt")
+    seeds = [3, 5, 700]
+    rest = np.setdiff1d(np.arange(n), seeds + [8])
+    sets = [[int(x) for x in rng.choice(rest, k, replace=False)] for _ in range(5)]
+    gh = cuda_lib.load_graph(g, model=model)
+    for theta in (1, 33, 400):
+        want = O.spread_sets(g, seeds, [8], sets, theta, 4, 1, model=model)
+        assert np.array_equal(cuda_lib.estimate_spread_sets(gh, seeds, [8], sets, theta, 4, 1), want)
+
+
+@pytest.mark.parametrize("deg", [1, 2, 3, 6])
+def test_non_tree_targets_few_and_many(cuda_lib, deg):
+    """Layered graphs whose samples have from a few hundred to several thousand non-tree edges:
+    both ways to resolve their targets, on the regular and the allocation-free entry point (whose
+    small slots hold neither the array nor the largest of these cascades)."""
+    rng = np.random.default_rng(deg)
+    layers, width = 12, 300
+    n = layers * width
+    src = np.concatenate([np.repeat(np.arange(i * width, (i + 1) * width), deg) for i in range(layers - 1)])
+    dst = (src // width + 1) * width + rng.integers(0, width, len(src))
+    keys = np.unique(src * n + dst)
+    g = _graph(n, keys // n, keys % n, 0.9)
+    gh = cuda_lib.load_graph(g)
+    seeds, blocked = list(range(0, width, 2)), [width + 1, 2 * width + 7]
+    want = O.decrease(g, seeds, blocked, 40, 6, 1)
+    assert np.array_equal(cuda_lib.estimate_decrease(gh, seeds, blocked, 40, 6, 1), want)
+    assert np.array_equal(cuda_lib.estimate_decrease_noalloc(gh, seeds, blocked, 40, 6, 1), want)
+
+
+@pytest.mark.parametrize("deg", [3, 5, 31, 32, 33, 130])
+def test_warp_tier_chunks(cuda_lib, deg):
+    """Frontier chunks of one and of many 32-group windows, with empty rows between full ones."""
+    rng = np.random.default_rng(deg)
+    n, hubs = 400, 40
+    src = np.repeat(np.arange(0, hubs), deg)
+    dst = rng.integers(0, n, len(src))
+    keys = np.unique((src * n + dst)[src != dst])
+    g = _graph(n, keys // n, keys % n, 0.15)
+    gh = cuda_lib.load_graph(g)
+    seeds = [0, 7, 390, 399]
+    for theta in (1, 500):
+        assert np.array_equal(cuda_lib.estimate_decrease(gh, seeds, [], theta, 3, 0),
+                              O.decrease(g, seeds, [], theta, 3, 0))
