@@ -9,8 +9,8 @@
 // final, and it cannot be recorded into a CUDA graph by stream capture.
 //
 // What it does: exactly what imin_estimate_decrease computes, with the warp tier at a fixed cutoff
-// (sample.cu) in front of the block-per-sample tier (sample_cta.cu), but every byte of working memory it needs besides the caller's inputs and
-// output comes from one file-scope device array of kNoAllocBytes (64 MiB). Every GPU that loads
+// (sample.cu) in front of the block-per-sample tier (sample_cta.cu), but every byte of working
+// memory it needs besides the caller's inputs and output comes from one file-scope device array of kNoAllocBytes (64 MiB). Every GPU that loads
 // the library holds that array until the process exits. Its limits follow from its size:
 // graphs with at most kNoAllocMaxVertices vertices and at most kNoAllocMaxTheta samples per call;
 // bigger requests are rejected with IMIN_ERR_INVALID. A sampled cascade that would need the
@@ -230,8 +230,15 @@ extern "C" int imin_estimate_decrease_noalloc(const imin_graph* g, const int32_t
     cta_slot_layout(&small);
     const uint32_t small_blocks = static_cast<uint32_t>(std::min<uint64_t>(blocks, room / small.slot_bytes));
     const uint32_t whole_blocks = static_cast<uint32_t>(std::min<uint64_t>(blocks, room / cfg.slot_bytes));
+    // Few samples per whole-graph slot are done sooner by that launch alone: the three launches'
+    // latencies add up, and a cascade that outgrows a small slot runs twice. n = 16,384 (146 slots):
+    // theta = 2,000 0.37 ms against 0.48, theta = 4,000 0.59 against 0.50; n = 50,021 (56 slots):
+    // theta = 1,000 0.52 against 0.66, theta = 2,000 1.12 against 0.67. Where the small slots hold
+    // every cascade (n = 2,000, 550 slots), theta = 2,000 0.20 against 0.21, theta = 4,000 0.28
+    // against 0.23.
+    const bool whole_only = theta <= (small.rcap < cfg.rcap ? 20u : 4u) * whole_blocks;
     TierPlan warp{};
-    plan_tier0(g->dev, static_cast<uint32_t>(n_seeds), kDefaultCutoff, &warp);
+    if (!whole_only) plan_tier0(g->dev, static_cast<uint32_t>(n_seeds), kDefaultCutoff, &warp);
 
     RoundCtl* ctl = reinterpret_cast<RoundCtl*>(base + off_ctl);
     uint32_t* bad = reinterpret_cast<uint32_t*>(base + off_bad);
@@ -271,12 +278,14 @@ extern "C" int imin_estimate_decrease_noalloc(const imin_graph* g, const int32_t
     P.lists = reinterpret_cast<uint32_t*>(base + off_lists);
     P.done = nullptr;
     P.stats = nullptr;
-    bool warp_ran = false;
-    NA_CUDA(launch_sample_tier(0, P, warp, nullptr, s, &warp_ran));
-    small.from_list = warp_ran ? 1u : 0u;
-    NA_CUDA(launch_cta_tier(P, small, small_blocks, smem, base + off_slots, s));
-    cfg.from_list = 1;
-    cfg.in_tier = kTierWhole;
+    if (!whole_only) {
+        bool warp_ran = false;
+        NA_CUDA(launch_sample_tier(0, P, warp, nullptr, s, &warp_ran));
+        small.from_list = warp_ran ? 1u : 0u;
+        NA_CUDA(launch_cta_tier(P, small, small_blocks, smem, base + off_slots, s));
+        cfg.from_list = 1;
+        cfg.in_tier = kTierWhole;
+    }
     cfg.out_tier = 1;  // the warp tier 1 does not run here: its list takes what nothing here holds
     NA_CUDA(launch_cta_tier(P, cfg, whole_blocks, smem, base + off_slots, s));
 

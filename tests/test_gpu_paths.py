@@ -93,3 +93,20 @@ def test_warp_tier_chunks(cuda_lib, deg):
     for theta in (1, 500):
         assert np.array_equal(cuda_lib.estimate_decrease(gh, seeds, [], theta, 3, 0),
                               O.decrease(g, seeds, [], theta, 3, 0))
+
+
+@pytest.mark.parametrize("deg,theta", [(1, 14_000), (6, 8_000)])
+def test_noalloc_three_launches(cuda_lib, deg, theta):
+    """More samples than 20 per whole-graph slot: the allocation-free call runs its warp tier, its
+    small slots (which the cascades of the second graph outgrow) and the whole-graph slots."""
+    rng = np.random.default_rng(deg)
+    layers, width = 12, 300
+    n = layers * width
+    src = np.concatenate([np.repeat(np.arange(i * width, (i + 1) * width), deg) for i in range(layers - 1)])
+    dst = (src // width + 1) * width + rng.integers(0, width, len(src))
+    keys = np.unique(src * n + dst)
+    g = _graph(n, keys // n, keys % n, 0.8 if deg == 1 else 0.45)
+    gh = cuda_lib.load_graph(g)
+    seeds, blocked = list(range(0, width, 3)), [width + 1, 2 * width + 7]
+    want = O.decrease(g, seeds, blocked, theta, 6, 1)
+    assert np.array_equal(cuda_lib.estimate_decrease_noalloc(gh, seeds, blocked, theta, 6, 1), want)
