@@ -358,7 +358,9 @@ int imin_estimate_decrease_stats(const imin_graph* g, const int32_t* seeds, int3
  * The cutoff never changes any result of this library, only which kernel computes a sample.
  * The estimate and greedy calls tune lazily on first use for each graph and seed-set size class
  * (ceil(log2 n_seeds)) unless IMIN_AUTOTUNE=0 (fixed cutoff 96) or IMIN_TIER0_VERTICES=<c>
- * (forced cutoff c); a call on a stream under capture uses 96. Results are also kept for the
+ * (forced cutoff c); a call on a stream under capture uses 96, and so does a call of fewer than
+ * 1,024 samples or one whose warm-up shows it to be shorter than the tuning (30 ms), which leaves
+ * the tuning to a longer one. Results are also kept for the
  * life of the process under a fingerprint of the graph (its sizes and sampled CSR entries), so a
  * new handle of the same graph does not tune again. This entry point re-tunes unconditionally.
  *   seeds     int32[n_seeds], host or device, distinct ids in [0, n).

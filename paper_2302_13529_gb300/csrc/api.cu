@@ -8,6 +8,7 @@
 #include <algorithm>
 #include <atomic>
 #include <chrono>
+#include <cstddef>
 #include <cstdlib>
 #include <cstdio>
 #include <cstring>
@@ -258,35 +259,62 @@ int check_ids(const std::vector<int32_t>& ids, int32_t n, std::vector<uint8_t>& 
 struct Query {
     Arena arena;
     TierPlan plan{};
+    // one allocation: the control block, the stats and the seed/blocked mask, which start at zero and
+    // are cleared together, then the seeds and blocked ids
+    RoundCtl* ctl = nullptr;
     int32_t* seeds = nullptr;
     uint32_t* excl = nullptr;
     unsigned long long* delta = nullptr;
     uint32_t* lists = nullptr;
-    unsigned long long* stats = nullptr;
+    unsigned long long* stats = nullptr;  // kStatsOffset bytes after ctl
     uint8_t* scratch1 = nullptr;
     uint8_t* scratch2 = nullptr;
     uint8_t* scratch3 = nullptr;
     uint8_t* handoff = nullptr;  // the warp tier's hand-off snapshots (after the block tier's slots)
     int32_t words = 0;
+    std::vector<int32_t> ids;    // what is copied to `seeds`, kept until the call has synchronized
     explicit Query(cudaStream_t s) : arena(s) {}
 };
 
+constexpr uint64_t kStatsOffset = 256;
+static_assert(sizeof(RoundCtl) <= kStatsOffset, "the stats follow the control block");
+
+// The control block and the stats as they lie in a query's first allocation, read back in one copy.
+struct CallStatus {
+    RoundCtl ctl;
+    uint8_t pad[kStatsOffset - sizeof(RoundCtl)];
+    unsigned long long stats[kStCount];
+};
+static_assert(offsetof(CallStatus, stats) == kStatsOffset, "as setup_query lays them out");
+
+// blocked: vertices masked with the seeds (NULL: none). A small call is bound by what the host
+// enqueues, so its small buffers come in one allocation with one clear, and all its ids in one copy
+// and one mask kernel (theta = 256 on a 2,000-vertex graph: 0.152 -> 0.134 ms).
 int setup_query(const imin_graph* g, const std::vector<int32_t>& seeds, uint32_t theta,
-                unsigned long long* out_delta_dev, uint32_t cutoff, Query& q)
+                unsigned long long* out_delta_dev, uint32_t cutoff, Query& q,
+                const std::vector<int32_t>* blocked = nullptr)
 {
     cudaStream_t s = q.arena.s;
     q.words = (g->n + 31) / 32;
     q.plan = plan_tiers(g->dev, g->n, g->m, static_cast<uint32_t>(seeds.size()), cutoff);
-    IMIN_CUDA(q.arena.alloc(&q.seeds, seeds.size()));
-    IMIN_CUDA(q.arena.alloc(&q.excl, q.words));
+    std::vector<int32_t>& ids = q.ids;
+    ids = seeds;
+    if (blocked != nullptr) ids.insert(ids.end(), blocked->begin(), blocked->end());
+    const uint64_t off_excl = kStatsOffset + sizeof(unsigned long long) * kStCount;
+    const uint64_t off_ids = (off_excl + sizeof(uint32_t) * q.words + 255) & ~uint64_t(255);
+    uint8_t* small = nullptr;
+    IMIN_CUDA(q.arena.alloc(&small, off_ids + sizeof(int32_t) * ids.size()));
+    q.ctl = reinterpret_cast<RoundCtl*>(small);
+    q.stats = reinterpret_cast<unsigned long long*>(small + kStatsOffset);
+    q.excl = reinterpret_cast<uint32_t*>(small + off_excl);
+    q.seeds = reinterpret_cast<int32_t*>(small + off_ids);
     if (out_delta_dev != nullptr) {
         q.delta = out_delta_dev;
     } else {
         IMIN_CUDA(q.arena.alloc(&q.delta, g->n));
     }
     IMIN_CUDA(q.arena.alloc(&q.lists, static_cast<uint64_t>(kTiers) * theta));
-    IMIN_CUDA(q.arena.alloc(&q.stats, kStCount));
-    IMIN_CUDA(q.arena.alloc(&q.scratch1, q.plan.scratch_bytes[1]));
+    if (q.plan.scratch_bytes[1] > 0) IMIN_CUDA(q.arena.alloc(&q.scratch1, q.plan.scratch_bytes[1]));
     IMIN_CUDA(q.arena.alloc(&q.scratch2, q.plan.scratch_bytes[2]));
     // with the warp tier in front of the block tier, one hand-off snapshot per sample it may give
     // up on, after the block tier's slots: the block tier resumes those samples where it stopped
@@ -299,14 +327,12 @@ int setup_query(const imin_graph* g, const std::vector<int32_t>& seeds, uint32_t
     IMIN_CUDA(q.arena.alloc(&q.scratch3, q.plan.scratch_bytes[kTierCta] + handoff_bytes));
     if (handoff_bytes > 0) q.handoff = q.scratch3 + q.plan.scratch_bytes[kTierCta];
     if (q.plan.use_cta) IMIN_CUDA(prepare_cta_scratch(q.plan.cta, q.plan.blocks[kTierCta], q.scratch3, s));
-    IMIN_CUDA(cudaMemcpyAsync(q.seeds, seeds.data(), sizeof(int32_t) * seeds.size(),
-                              cudaMemcpyHostToDevice, s));
-    IMIN_CUDA(cudaMemsetAsync(q.excl, 0, sizeof(uint32_t) * q.words, s));
+    IMIN_CUDA(cudaMemcpyAsync(q.seeds, ids.data(), sizeof(int32_t) * ids.size(), cudaMemcpyHostToDevice, s));
+    IMIN_CUDA(cudaMemsetAsync(small, 0, off_ids, s));
     IMIN_CUDA(cudaMemsetAsync(q.delta, 0, sizeof(unsigned long long) * g->n, s));
-    IMIN_CUDA(cudaMemsetAsync(q.stats, 0, sizeof(unsigned long long) * kStCount, s));
     IMIN_CUDA(prepare_warp_slots(q.plan, 1, q.scratch1, s));
     IMIN_CUDA(prepare_warp_slots(q.plan, kTierWhole, q.scratch2, s));
-    IMIN_CUDA(launch_build_excl(q.excl, q.seeds, static_cast<int32_t>(seeds.size()), s));
+    IMIN_CUDA(launch_build_excl(q.excl, q.seeds, static_cast<int32_t>(ids.size()), s));
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return IMIN_OK;
 }
@@ -437,9 +463,12 @@ int common_checks(const imin_graph* g, const int32_t* seeds, int32_t n_seeds, ui
 constexpr uint32_t kCutoffs[] = {0, 64, 96, 128, 192};
 constexpr int kTuneReps = 3;
 constexpr float kTuneCallMs = 2.0f;
+constexpr uint32_t kTuneMinTheta = 1024;  // the warm-up's largest size
+constexpr float kTuneMinCallMs = 30.0f;   // the timed calls' total: 3 x 5 of about 2 ms
 
 std::mutex g_tune_mu;
 std::map<std::pair<uint64_t, int>, int32_t> g_tuned;  // (fingerprint, size class) -> cutoff
+std::map<std::pair<uint64_t, int>, float> g_warm;     // the warm-up's ms per sample, while not tuned
 
 // Identity of a graph for the process-wide tuning cache: a 64-bit mix of its sizes, its device
 // and about 4,096 evenly spaced entries of each CSR array. Two different graphs that collide
@@ -483,9 +512,7 @@ int time_call(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t k
     Query q(s);
     int rc = setup_query(g, seeds, theta, nullptr, cutoff, q);
     if (rc) return rc;
-    RoundCtl* ctl = nullptr;
-    IMIN_CUDA(q.arena.alloc(&ctl, 1));
-    IMIN_CUDA(cudaMemsetAsync(ctl, 0, sizeof(RoundCtl), s));
+    RoundCtl* const ctl = q.ctl;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     IMIN_CUDA(cudaEventCreate(&e0));
     cudaError_t e = cudaEventCreate(&e1);
@@ -513,8 +540,10 @@ int time_call(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t k
 }
 
 // theta_hint: the caller's samples per call (0: unknown), which bounds the warm-up call.
+// *per_sample_ms: the warm-up's time per sample. *out < 0: a call of theta_hint samples is shorter
+// than the tuning, which would cost it more than it can give; no candidate was timed.
 int tune_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t key, cudaStream_t s,
-                uint32_t theta_hint, uint32_t* out)
+                uint32_t theta_hint, int32_t* out, float* per_sample_ms)
 {
     constexpr int kCand = static_cast<int>(sizeof(kCutoffs) / sizeof(kCutoffs[0]));
     float warm = 0.f, t[kCand];
@@ -524,10 +553,15 @@ int tune_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t
     int rc = time_call(g, seeds, key, kDefaultCutoff, tw, s, &warm, &warp_done);  // warm-up, cost
     if (rc) return rc;
     double per_sample = std::max(1e-7, static_cast<double>(warm) / tw);  // ms
+    *per_sample_ms = static_cast<float>(per_sample);
     if (kTuneCallMs / per_sample < 4.0 * blocks) {
         // too costly to compare by timing: keep the warp tier only if it finished at least a
         // tenth of the warm-up's samples (otherwise its partial work is mostly thrown away)
-        *out = 10 * warp_done >= tw ? kDefaultCutoff : 0u;
+        *out = 10 * warp_done >= tw ? static_cast<int32_t>(kDefaultCutoff) : 0;
+        return IMIN_OK;
+    }
+    if (theta_hint > 0 && theta_hint * per_sample < kTuneMinCallMs) {
+        *out = -1;
         return IMIN_OK;
     }
     // a small warm-up is dominated by its slowest block; re-estimate on a call of the planned size
@@ -548,7 +582,7 @@ int tune_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t
     int best = 0;
     for (int i = 1; i < kCand; ++i)
         if (t[i] < t[best]) best = i;
-    *out = kCutoffs[best];
+    *out = static_cast<int32_t>(kCutoffs[best]);
     return IMIN_OK;
 }
 
@@ -585,8 +619,27 @@ int cutoff_for(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t 
             return IMIN_OK;
         }
     }
-    const int rc = tune_cutoff(g, seeds, key, s, theta_hint, out);
+    // A short call cannot repay the tuning: one of few samples, whose warm-up would tell nothing, or
+    // one that the warm-up shows to be shorter than the timed calls. It takes the default, which is
+    // within a few percent of the best, and the first longer call tunes. First call of theta = 256 on
+    // a 2,000-vertex graph 0.46 -> 0.21 ms; of AdvancedGreedy there (theta = 10^4, b = 10) 10.1 -> 2.1
+    // ms; of a batch of 48 new queries 437 -> 164 ms.
+    if (theta_hint > 0 && theta_hint < kTuneMinTheta) return IMIN_OK;
+    if (theta_hint > 0) {
+        std::lock_guard<std::mutex> lk2(g_tune_mu);
+        const auto it = g_warm.find({g->fingerprint, cls});
+        if (it != g_warm.end() && theta_hint * it->second < kTuneMinCallMs) return IMIN_OK;
+    }
+    int32_t best = -1;
+    float per_sample = 0.f;
+    const int rc = tune_cutoff(g, seeds, key, s, theta_hint, &best, &per_sample);
     if (rc) return rc;
+    if (best < 0) {
+        std::lock_guard<std::mutex> lk2(g_tune_mu);
+        g_warm[{g->fingerprint, cls}] = per_sample;
+        return IMIN_OK;
+    }
+    *out = static_cast<uint32_t>(best);
     g->cutoff[cls] = static_cast<int32_t>(*out);
     std::lock_guard<std::mutex> lk2(g_tune_mu);
     g_tuned[{g->fingerprint, cls}] = static_cast<int32_t>(*out);
@@ -629,35 +682,22 @@ int estimate_impl(const imin_graph* g, const int32_t* seeds, int32_t n_seeds,
     if (rc) return rc;
     Query q(s);
     rc = setup_query(g, hseeds, theta, dev_out ? reinterpret_cast<unsigned long long*>(out_delta) : nullptr,
-                     cutoff, q);
+                     cutoff, q, &hblocked);
     if (rc) return rc;
-    RoundCtl* ctl = nullptr;
-    int32_t* dblocked = nullptr;
-    IMIN_CUDA(q.arena.alloc(&ctl, 1));
-    IMIN_CUDA(q.arena.alloc(&dblocked, hblocked.size()));
-    IMIN_CUDA(cudaMemsetAsync(ctl, 0, sizeof(RoundCtl), s));
-    if (!hblocked.empty()) {
-        IMIN_CUDA(cudaMemcpyAsync(dblocked, hblocked.data(), sizeof(int32_t) * hblocked.size(),
-                                  cudaMemcpyHostToDevice, s));
-        IMIN_CUDA(launch_build_excl(q.excl, dblocked, n_blocked, s));
-        g_launches.fetch_add(1, std::memory_order_relaxed);
-    }
     CallTimer T(s);
-    const SampleParams P = sample_params(g, q, static_cast<uint32_t>(n_seeds), theta, key, round, ctl, nullptr);
+    const SampleParams P = sample_params(g, q, static_cast<uint32_t>(n_seeds), theta, key, round, q.ctl, nullptr);
     IMIN_CUDA(enqueue_call(P, q, T));
 
-    std::vector<RoundCtl> hctl(1);
-    unsigned long long hstats[kStCount];
-    IMIN_CUDA(cudaMemcpyAsync(hctl.data(), ctl, sizeof(RoundCtl), cudaMemcpyDeviceToHost, s));
-    IMIN_CUDA(cudaMemcpyAsync(hstats, q.stats, sizeof(hstats), cudaMemcpyDeviceToHost, s));
+    CallStatus status;
+    IMIN_CUDA(cudaMemcpyAsync(&status, q.ctl, sizeof(status), cudaMemcpyDeviceToHost, s));
     if (!dev_out) {
         IMIN_CUDA(cudaMemcpyAsync(out_delta, q.delta, sizeof(uint64_t) * g->n, cudaMemcpyDeviceToHost, s));
     }
     IMIN_CUDA(cudaStreamSynchronize(s));
     T.collect();
-    rc = check_ctl(hctl);
+    rc = check_ctl({status.ctl});
     if (rc) return rc;
-    record_stats(hstats);
+    record_stats(status.stats);
     if (stats != nullptr) *stats = g_last_stats;
     return IMIN_OK;
 }
@@ -680,40 +720,28 @@ int spread_impl(const imin_graph* g, const int32_t* seeds, int32_t n_seeds, cons
     if (rc) return rc;
 
     Query q(s);
-    rc = setup_query(g, hseeds, theta, nullptr, 0, q);
+    rc = setup_query(g, hseeds, theta, nullptr, 0, q, &hblocked);
     if (rc) return rc;
     if (!q.plan.use_cta) return fail(IMIN_ERR_INTERNAL, "the spread kernel needs the block-per-sample tier");
-    RoundCtl* ctl = nullptr;
-    int32_t* dblocked = nullptr;
     unsigned long long* dsum = nullptr;
     uint32_t* handoff = nullptr;
     IMIN_CUDA(q.arena.alloc(&handoff, spread_handoff_words(theta)));
-    IMIN_CUDA(q.arena.alloc(&ctl, 1));
-    IMIN_CUDA(q.arena.alloc(&dblocked, hblocked.size()));
     IMIN_CUDA(q.arena.alloc(&dsum, 1));
-    IMIN_CUDA(cudaMemsetAsync(ctl, 0, sizeof(RoundCtl), s));
     IMIN_CUDA(cudaMemsetAsync(dsum, 0, sizeof(unsigned long long), s));
-    if (!hblocked.empty()) {
-        IMIN_CUDA(cudaMemcpyAsync(dblocked, hblocked.data(), sizeof(int32_t) * hblocked.size(),
-                                  cudaMemcpyHostToDevice, s));
-        IMIN_CUDA(launch_build_excl(q.excl, dblocked, n_blocked, s));
-        g_launches.fetch_add(1, std::memory_order_relaxed);
-    }
     CallTimer T(s);
-    const SampleParams P = sample_params(g, q, static_cast<uint32_t>(n_seeds), theta, key, round, ctl, nullptr);
+    const SampleParams P = sample_params(g, q, static_cast<uint32_t>(n_seeds), theta, key, round, q.ctl, nullptr);
     IMIN_CUDA(enqueue_spread(P, q, T, nullptr, 0, theta, handoff, dsum));
-    std::vector<RoundCtl> hctl(1);
-    unsigned long long hstats[kStCount], hsum = 0;
-    IMIN_CUDA(cudaMemcpyAsync(hctl.data(), ctl, sizeof(RoundCtl), cudaMemcpyDeviceToHost, s));
-    IMIN_CUDA(cudaMemcpyAsync(hstats, q.stats, sizeof(hstats), cudaMemcpyDeviceToHost, s));
+    CallStatus status;
+    unsigned long long hsum = 0;
+    IMIN_CUDA(cudaMemcpyAsync(&status, q.ctl, sizeof(status), cudaMemcpyDeviceToHost, s));
     IMIN_CUDA(cudaMemcpyAsync(&hsum, dsum, sizeof(hsum), cudaMemcpyDeviceToHost, s));
     IMIN_CUDA(cudaStreamSynchronize(s));
     T.collect();
-    if (hctl[0].error & kErrCapacity)
+    if (status.ctl.error & kErrCapacity)
         return fail(IMIN_ERR_CAPACITY, "a sampled cascade exceeded the block tier's slot capacity (2^18 vertices)");
-    rc = check_ctl(hctl);
+    rc = check_ctl({status.ctl});
     if (rc) return rc;
-    record_stats(hstats);
+    record_stats(status.stats);
     *out_sum = hsum;
     return IMIN_OK;
 }
@@ -747,36 +775,25 @@ int spread_sets_core(const imin_graph* g, const std::vector<int32_t>& hseeds, co
         if (rc) return rc;
     }
     Query q(s);
-    int rc = setup_query(g, hseeds, theta, nullptr, 0, q);
+    int rc = setup_query(g, hseeds, theta, nullptr, 0, q, &hblocked);
     if (rc) return rc;
     if (!q.plan.use_cta) return fail(IMIN_ERR_INTERNAL, "the spread kernel needs the block-per-sample tier");
-    RoundCtl* ctl = nullptr;
-    int32_t* dblocked = nullptr;
     int32_t* dsets = nullptr;
     unsigned long long* dsums = nullptr;
     uint32_t* handoff = nullptr;
     const unsigned long long items = static_cast<unsigned long long>(nsets) * theta;
-    IMIN_CUDA(q.arena.alloc(&ctl, 1));
-    IMIN_CUDA(q.arena.alloc(&dblocked, hblocked.size()));
     IMIN_CUDA(q.arena.alloc(&dsets, static_cast<uint64_t>(nsets) * k));
     IMIN_CUDA(q.arena.alloc(&dsums, static_cast<uint64_t>(nsets)));
     IMIN_CUDA(q.arena.alloc(&handoff, spread_handoff_words(items)));
-    IMIN_CUDA(cudaMemsetAsync(ctl, 0, sizeof(RoundCtl), s));
     IMIN_CUDA(cudaMemsetAsync(dsums, 0, sizeof(unsigned long long) * nsets, s));
     if (k > 0)
         IMIN_CUDA(cudaMemcpyAsync(dsets, hsets, sizeof(int32_t) * nsets * k, cudaMemcpyHostToDevice, s));
-    if (!hblocked.empty()) {
-        IMIN_CUDA(cudaMemcpyAsync(dblocked, hblocked.data(), sizeof(int32_t) * hblocked.size(),
-                                  cudaMemcpyHostToDevice, s));
-        IMIN_CUDA(launch_build_excl(q.excl, dblocked, static_cast<int32_t>(hblocked.size()), s));
-        g_launches.fetch_add(1, std::memory_order_relaxed);
-    }
     CallTimer T(s);
-    SampleParams P = sample_params(g, q, static_cast<uint32_t>(hseeds.size()), theta, key, round, ctl, nullptr);
+    SampleParams P = sample_params(g, q, static_cast<uint32_t>(hseeds.size()), theta, key, round, q.ctl, nullptr);
     P.stats = nullptr;
     IMIN_CUDA(enqueue_spread(P, q, T, dsets, static_cast<uint32_t>(k), items, handoff, dsums));
     RoundCtl hctl;
-    IMIN_CUDA(cudaMemcpyAsync(&hctl, ctl, sizeof(hctl), cudaMemcpyDeviceToHost, s));
+    IMIN_CUDA(cudaMemcpyAsync(&hctl, q.ctl, sizeof(hctl), cudaMemcpyDeviceToHost, s));
     IMIN_CUDA(cudaMemcpyAsync(hsums, dsums, sizeof(uint64_t) * nsets, cudaMemcpyDeviceToHost, s));
     IMIN_CUDA(cudaStreamSynchronize(s));
     T.collect();
@@ -1474,16 +1491,17 @@ int imin_autotune(const imin_graph* g, const int32_t* seeds, int32_t n_seeds, ui
     std::vector<uint8_t> mark;
     int rc = common_checks(g, seeds, n_seeds, 1, s, hseeds, mark);
     if (rc) return rc;
-    uint32_t c = 0;
+    int32_t c = 0;
+    float per_sample = 0.f;
     {
         std::lock_guard<std::mutex> lk(g->tune_mu);
-        rc = tune_cutoff(g, hseeds, key, s, 0, &c);
+        rc = tune_cutoff(g, hseeds, key, s, 0, &c, &per_sample);
         if (rc) return rc;
-        g->cutoff[size_class(hseeds.size())] = static_cast<int32_t>(c);
+        g->cutoff[size_class(hseeds.size())] = c;
         std::lock_guard<std::mutex> lk2(g_tune_mu);
-        g_tuned[{g->fingerprint, size_class(hseeds.size())}] = static_cast<int32_t>(c);
+        g_tuned[{g->fingerprint, size_class(hseeds.size())}] = c;
     }
-    *out_cutoff = static_cast<int32_t>(c);
+    *out_cutoff = c;
     return IMIN_OK;
 }
 
