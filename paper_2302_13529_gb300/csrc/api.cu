@@ -623,7 +623,7 @@ int cutoff_for(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t 
     // one that the warm-up shows to be shorter than the timed calls. It takes the default, which is
     // within a few percent of the best, and the first longer call tunes. First call of theta = 256 on
     // a 2,000-vertex graph 0.46 -> 0.21 ms; of AdvancedGreedy there (theta = 10^4, b = 10) 10.1 -> 2.1
-    // ms; of a batch of 48 new queries 437 -> 164 ms.
+    // ms; of a batch of 48 new queries 467 -> 52 ms.
     if (theta_hint > 0 && theta_hint < kTuneMinTheta) return IMIN_OK;
     if (theta_hint > 0) {
         std::lock_guard<std::mutex> lk2(g_tune_mu);
