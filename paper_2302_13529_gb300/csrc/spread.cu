@@ -255,6 +255,12 @@ k_spread_block(SampleParams P, CtaCfg C, SpreadWork W)
         if (sh.item >= count) break;
         const uint32_t* h = W.handoff + static_cast<uint64_t>(sh.item) * kHandoffWords;
         const uint32_t set = h[0], at = h[2], found = P.ns + h[3];
+        // a slot of a large graph holds at most 2^18 ids, and the warp left the vertices it could not
+        // queue for the block to find: a cascade that does not fit already will not fit later
+        if (1 + found > C.rcap) {
+            if (tid == 0) atomicOr(&P.ctl->error, kErrCapacity);
+            continue;
+        }
         // slot ids start at 1, as in Alg. 2's slots
         for (uint32_t i = tid; i < found; i += kCtaThreads) {
             const uint32_t v = i < P.ns ? static_cast<uint32_t>(P.seeds[i]) : h[kHeader + i - P.ns];

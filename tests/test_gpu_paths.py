@@ -110,3 +110,45 @@ def test_noalloc_three_launches(cuda_lib, deg, theta):
     seeds, blocked = list(range(0, width, 3)), [width + 1, 2 * width + 7]
     want = O.decrease(g, seeds, blocked, theta, 6, 1)
     assert np.array_equal(cuda_lib.estimate_decrease_noalloc(gh, seeds, blocked, theta, 6, 1), want)
+
+
+BIG = (1 << 18) + 40  # above 2^18 vertices: the visited bitmap is in the block's slot, whose ids are capped
+
+
+def _big_star(leaves, seeds, p=1.0):
+    """Seed 0 -> `leaves` vertices, the other seeds without edges, on a graph of BIG vertices."""
+    dst = list(range(seeds, seeds + leaves))
+    return _graph(BIG, [0] * leaves, dst, p)
+
+
+@pytest.mark.parametrize("seeds", [1, 30, 300])
+@pytest.mark.parametrize("room", [-300, -90, -2, -1, 0, 1])
+def test_resumed_spread_cascade_against_the_slot_capacity(cuda_lib, monkeypatch, seeds, room):
+    """257 leaves, one more than the warp kernel's queue: every cascade is handed over with the seeds
+    and 256 leaves and needs 1 + |S| + 257 ids. A slot of fewer reports the capacity error, whether
+    the hand-off itself fits it (room -1) or not; one of just as many gives the exact sum."""
+    g = _big_star(257, seeds)
+    gh = cuda_lib.load_graph(g)
+    monkeypatch.setenv("IMIN_CTA_VERTEX_CAP", str(max(1 + seeds + 257 + room, 2)))
+    s = list(range(seeds))
+    if room < 0:
+        for call in (lambda: cuda_lib.estimate_spread(gh, s, [], 40, 9, 2),
+                     lambda: cuda_lib.estimate_spread_sets(gh, s, [], [[BIG - 1]], 40, 9, 2)):
+            with pytest.raises(cuda_lib.IminError) as ei:
+                call()
+            assert ei.value.code == -4  # IMIN_ERR_CAPACITY
+    else:
+        assert cuda_lib.estimate_spread(gh, s, [], 40, 9, 2) == 40 * (seeds + 257)
+
+
+@pytest.mark.parametrize("seeds,k", [(1, 3), (300, 1), (300, 64)])
+def test_spread_sets_handed_over_on_a_large_graph(cuda_lib, seeds, k):
+    """Blocker sets whose cascades outgrow the warp kernel on a graph with its bitmap in global memory,
+    with few and with more than 256 seeds: the set's vertices stay blocked after the hand-off."""
+    g = _big_star(400, seeds, 0.9)
+    gh = cuda_lib.load_graph(g)
+    s = list(range(seeds))
+    rng = np.random.default_rng(k)
+    sets = [[int(x) for x in seeds + rng.choice(400, k, replace=False)] for _ in range(3)]
+    want = O.spread_sets(g, s, [seeds + 400], sets, 50, 4, 1)
+    assert np.array_equal(cuda_lib.estimate_spread_sets(gh, s, [seeds + 400], sets, 50, 4, 1), want)
