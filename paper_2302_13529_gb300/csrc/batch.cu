@@ -158,9 +158,10 @@ __global__ void __launch_bounds__(cta_threads<kSmemBitmap>(), 1024 / cta_threads
             const uint32_t j = hdr[0], q = hdr[8];
             const SampleParams P = params_of(B.q[q], B.step - B.q[q].start);
             uint32_t from[3];
-            restore_handoff<kCtaThreads>(P, hb, S, bm, sh, tid, from);
-            const int rc = run_sample_cta<kSmemBitmap, false, M>(P, C, bm, dsm, sh, S, j, tid, sc, examined, live,
-                                                                 ExtraBlocked{nullptr, 0u}, from);
+            int rc = kSampleOverflow;
+            if (restore_handoff<kCtaThreads>(P, C, hb, S, bm, sh, tid, from))
+                rc = run_sample_cta<kSmemBitmap, false, M>(P, C, bm, dsm, sh, S, j, tid, sc, examined, live,
+                                                           ExtraBlocked{nullptr, 0u}, from);
             if (tid == 0) {
                 if (rc == kSampleOverflow) {
                     const uint32_t p = atomicAdd(&B.ctl->over_count, 1u);

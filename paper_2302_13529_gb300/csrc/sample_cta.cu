@@ -56,9 +56,10 @@ __global__ void __launch_bounds__(cta_threads<kSmemBitmap>(), 1024 / cta_threads
             const uint8_t* hb = C.scratch + static_cast<uint64_t>(gridDim.x) * C.slot_bytes +
                                 static_cast<uint64_t>(sh.item) * C.handoff_stride;
             uint32_t from[3];
-            restore_handoff<kCtaThreads>(P, hb, S, bm, sh, tid, from);
-            rc = run_sample_cta<kSmemBitmap, false, M>(P, C, bm, dsm, sh, S, j, tid, sc, examined, live,
-                                                       ExtraBlocked{nullptr, 0u}, from);
+            rc = kSampleOverflow;
+            if (restore_handoff<kCtaThreads>(P, C, hb, S, bm, sh, tid, from))
+                rc = run_sample_cta<kSmemBitmap, false, M>(P, C, bm, dsm, sh, S, j, tid, sc, examined, live,
+                                                           ExtraBlocked{nullptr, 0u}, from);
         } else {
             rc = run_sample_cta<kSmemBitmap, false, M>(P, C, bm, dsm, sh, S, j, tid, sc, examined, live);
         }

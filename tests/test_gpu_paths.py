@@ -152,3 +152,44 @@ def test_spread_sets_handed_over_on_a_large_graph(cuda_lib, seeds, k):
     sets = [[int(x) for x in seeds + rng.choice(400, k, replace=False)] for _ in range(3)]
     want = O.spread_sets(g, s, [seeds + 400], sets, 50, 4, 1)
     assert np.array_equal(cuda_lib.estimate_spread_sets(gh, s, [seeds + 400], sets, 50, 4, 1), want)
+
+
+@pytest.mark.parametrize("cap", [2, 64, 101, 130, 1000])
+@pytest.mark.parametrize("seeds,cutoff", [(100, "0"), (30, "0"), (30, "96"), (30, "192")])
+def test_start_of_a_sample_against_the_slot_capacity(cuda_lib, monkeypatch, cap, seeds, cutoff):
+    """A slot that cannot hold the seeds, or the vertices a warp found before it gave up, leaves the
+    sample to the whole-graph tier: counters, blockers and the batched blockers stay the oracle's."""
+    src = np.repeat(np.arange(400), 4)
+    dst = np.random.default_rng(5).integers(0, 400, len(src))
+    keys = np.unique((src * BIG + dst)[src != dst])
+    g = _graph(BIG, keys // BIG, keys % BIG, 0.4)
+    monkeypatch.setenv("IMIN_CTA_VERTEX_CAP", str(cap))
+    monkeypatch.setenv("IMIN_TIER0_VERTICES", cutoff)
+    gh = cuda_lib.load_graph(g)
+    s = list(range(0, 2 * seeds, 2))
+    got, st = cuda_lib.estimate_decrease(gh, s, [399], 60, 3, 1, stats=True)
+    assert np.array_equal(got, O.decrease(g, s, [399], 60, 3, 1))
+    assert sum(st["tier_samples"]) == 60
+    if cap <= seeds:
+        assert st["tier_samples"][3] == 0
+    want = O.advanced_greedy(g, s, 2, 60, 3)
+    assert np.array_equal(cuda_lib.advanced_greedy(gh, s, 2, 60, 3), want)
+    assert np.array_equal(cuda_lib.batch_advanced_greedy([(gh, s, 2, 60, 3)])[0], want)
+
+
+@pytest.mark.parametrize("edges", ["1", "3", "20"])
+def test_non_tree_edges_of_a_hand_off_against_the_slot_capacity(cuda_lib, monkeypatch, edges):
+    """Block-tier slots of fewer non-tree edges than the warp tier holds (48 at cutoff 192)."""
+    src = np.repeat(np.arange(500), 6)
+    dst = np.random.default_rng(6).integers(0, 500, len(src))
+    keys = np.unique((src * 500 + dst)[src != dst])
+    g = _graph(500, keys // 500, keys % 500, 0.25)
+    monkeypatch.setenv("IMIN_CTA_EDGE_CAP", edges)
+    monkeypatch.setenv("IMIN_TIER0_VERTICES", "192")
+    gh = cuda_lib.load_graph(g)
+    s = [0, 7, 14, 21]
+    got, st = cuda_lib.estimate_decrease(gh, s, [], 3000, 3, 1, stats=True)
+    assert np.array_equal(got, O.decrease(g, s, [], 3000, 3, 1))
+    assert sum(st["tier_samples"]) == 3000 and st["tier_samples"][2] > 0
+    want = O.advanced_greedy(g, s, 2, 500, 3)
+    assert np.array_equal(cuda_lib.batch_advanced_greedy([(gh, s, 2, 500, 3)])[0], want)
