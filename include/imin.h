@@ -353,14 +353,14 @@ int imin_estimate_decrease_stats(const imin_graph* g, const int32_t* seeds, int3
  * {0, 64, 96, 128, 192} (0 = block tier only), interleaved, and keeps the candidate with the
  * smallest minimum time. When fewer than 4 samples per block fit in 2 ms (huge cascades), it does
  * not time the candidates: it keeps 96 if the warm-up's warp tier finished at least a tenth of
- * its samples, and 0 otherwise. The first warm-up call samples at most 1,024 graphs (at most the caller's
- * theta for the lazy tuning).
+ * its samples, and 0 otherwise. The first warm-up call samples 1,024 graphs.
  * The cutoff never changes any result of this library, only which kernel computes a sample.
- * The estimate and greedy calls tune lazily on first use for each graph and seed-set size class
+ * The estimate and greedy calls tune lazily for each graph and seed-set size class
  * (ceil(log2 n_seeds)) unless IMIN_AUTOTUNE=0 (fixed cutoff 96) or IMIN_TIER0_VERTICES=<c>
- * (forced cutoff c); a call on a stream under capture uses 96, and so does a call of fewer than
- * 1,024 samples or one whose warm-up shows it to be shorter than the tuning (30 ms), which leaves
- * the tuning to a longer one. Results are also kept for the
+ * (forced cutoff c); a call on a stream under capture uses 96. The samples of the calls on a graph
+ * and class (b * theta of a greedy call) are added up: the first warm-up runs at 1,024, and the
+ * candidates are timed when the sum comes to 16 times the samples of the timed calls (at most
+ * 16 * 15 * 65,536). Until then calls use 96. Results and sums are kept for the
  * life of the process under a fingerprint of the graph (its sizes and sampled CSR entries), so a
  * new handle of the same graph does not tune again. This entry point re-tunes unconditionally.
  *   seeds     int32[n_seeds], host or device, distinct ids in [0, n).

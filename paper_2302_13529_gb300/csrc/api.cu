@@ -452,10 +452,10 @@ int common_checks(const imin_graph* g, const int32_t* seeds, int32_t n_seeds, ui
 // hits all of them alike; the candidate with the smallest minimum time wins. Each call samples
 // 24 graphs per resident block of the block tier (at least 8,192, at most 65,536), so that the
 // end of a call -- blocks finishing their last cascades at different times -- does not decide
-// the comparison. The cost is bounded: the warm-up call samples at most as many graphs as the
-// caller asked for (and at most 1,024); from its time per sample, each timed call is sized to
-// take about kTuneCallMs, and when fewer than 4 samples per block would fit in that time (graphs
-// whose cascades are huge, where the cutoff hardly matters) the default is kept untimed. The
+// the comparison. The cost is bounded: the warm-up call samples 1,024 graphs; from its time per
+// sample, each timed call is sized to take about kTuneCallMs, and when fewer than 4 samples per block
+// would fit in that time (graphs whose cascades are huge, where the cutoff hardly matters) none is
+// timed. Calls that come before the tuning has been earned (kTuneRepay) take the default. The
 // choice never changes a result -- only which tier computes each sample -- and is cached per
 // graph handle and seed-set size class, and process-wide under the graph's fingerprint, so that
 // a new handle of the same graph reuses it.
@@ -463,12 +463,20 @@ int common_checks(const imin_graph* g, const int32_t* seeds, int32_t n_seeds, ui
 constexpr uint32_t kCutoffs[] = {0, 64, 96, 128, 192};
 constexpr int kTuneReps = 3;
 constexpr float kTuneCallMs = 2.0f;
-constexpr uint32_t kTuneMinTheta = 1024;  // the warm-up's largest size
-constexpr float kTuneMinCallMs = 30.0f;   // the timed calls' total: 3 x 5 of about 2 ms
+constexpr uint32_t kTuneWarmup = 1024;    // samples of the warm-up call
+constexpr uint64_t kTuneRepay = 16;       // samples drawn per sample the tuner times (cutoff_for)
+constexpr size_t kUntunedMax = 4096;      // entries of g_untuned
+
+// A graph and size class that is not tuned yet: the samples that its calls have drawn, and how many
+// they have to draw before the tuner looks at it (again).
+struct Untuned {
+    uint64_t samples = 0;
+    uint64_t need = kTuneWarmup;
+};
 
 std::mutex g_tune_mu;
 std::map<std::pair<uint64_t, int>, int32_t> g_tuned;  // (fingerprint, size class) -> cutoff
-std::map<std::pair<uint64_t, int>, float> g_warm;     // the warm-up's ms per sample, while not tuned
+std::map<std::pair<uint64_t, int>, Untuned> g_untuned;
 
 // Identity of a graph for the process-wide tuning cache: a 64-bit mix of its sizes, its device
 // and about 4,096 evenly spaced entries of each CSR array. Two different graphs that collide
@@ -539,38 +547,46 @@ int time_call(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t k
     return check_ctl(hctl);
 }
 
-// theta_hint: the caller's samples per call (0: unknown), which bounds the warm-up call.
-// *per_sample_ms: the warm-up's time per sample. *out < 0: a call of theta_hint samples is shorter
-// than the tuning, which would cost it more than it can give; no candidate was timed.
+// drawn: samples that the calls so far have drawn on this graph (0: tune in any case). *out < 0: they
+// have not earned the tuning yet (its timed calls are more than a kTuneRepay-th of them); no candidate
+// was timed, and *need is the number of samples that will.
 int tune_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t key, cudaStream_t s,
-                uint32_t theta_hint, int32_t* out, float* per_sample_ms)
+                uint64_t drawn, int32_t* out, uint64_t* need)
 {
     constexpr int kCand = static_cast<int>(sizeof(kCutoffs) / sizeof(kCutoffs[0]));
     float warm = 0.f, t[kCand];
     const uint32_t blocks = cta_blocks(g, seeds.size());
-    const uint32_t tw = std::max<uint32_t>(1, std::min<uint32_t>(1024, theta_hint ? theta_hint : 1024));
+    const uint32_t tw = kTuneWarmup;
     unsigned long long warp_done = 0;
     int rc = time_call(g, seeds, key, kDefaultCutoff, tw, s, &warm, &warp_done);  // warm-up, cost
     if (rc) return rc;
+    const auto costly = [&] { return kTuneCallMs * tw < 4.0 * blocks * warm; };
+    if (costly()) {  // once more: a process's first call also waits for its kernels to be loaded
+        rc = time_call(g, seeds, key, kDefaultCutoff, tw, s, &warm, &warp_done);
+        if (rc) return rc;
+    }
     double per_sample = std::max(1e-7, static_cast<double>(warm) / tw);  // ms
-    *per_sample_ms = static_cast<float>(per_sample);
-    if (kTuneCallMs / per_sample < 4.0 * blocks) {
+    if (costly()) {
         // too costly to compare by timing: keep the warp tier only if it finished at least a
         // tenth of the warm-up's samples (otherwise its partial work is mostly thrown away)
         *out = 10 * warp_done >= tw ? static_cast<int32_t>(kDefaultCutoff) : 0;
         return IMIN_OK;
     }
-    if (theta_hint > 0 && theta_hint * per_sample < kTuneMinCallMs) {
+    const auto too_early = [&](uint32_t timed) {
         *out = -1;
-        return IMIN_OK;
-    }
-    // a small warm-up is dominated by its slowest block; re-estimate on a call of the planned size
+        *need = kTuneRepay * kTuneReps * kCand * timed;
+        return drawn > 0 && drawn < *need;
+    };
+    // a small warm-up is dominated by its slowest block, so the timed calls will have at least the
+    // samples it makes room for; re-estimate on a call of that size
     uint32_t theta = static_cast<uint32_t>(std::min<double>({kTuneCallMs / per_sample, 24.0 * blocks, 65536.0}));
+    if (too_early(theta)) return IMIN_OK;
     rc = time_call(g, seeds, key, kDefaultCutoff, theta, s, &warm);
     if (rc) return rc;
     per_sample = std::max(1e-7, static_cast<double>(warm) / theta);
     theta = static_cast<uint32_t>(std::min<double>({std::max(kTuneCallMs / per_sample, 4.0 * blocks),
                                                     24.0 * blocks, 65536.0}));
+    if (too_early(theta)) return IMIN_OK;
     for (int rep = 0; rep < kTuneReps; ++rep) {
         for (int i = 0; i < kCand; ++i) {
             float ms = 0.f;
@@ -588,8 +604,9 @@ int tune_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t
 
 // The cutoff for a call: IMIN_TIER0_VERTICES forces one; IMIN_AUTOTUNE=0, or a stream being
 // captured (the tuner synchronizes), gives the default; otherwise the tuned value, tuning on first
-// use for this graph and seed-set size class.
-int cutoff_for(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t key, uint32_t theta_hint,
+// use for this graph and seed-set size class, once its calls have drawn enough samples. samples: what
+// this call draws over all its rounds.
+int cutoff_for(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t key, uint64_t samples,
                cudaStream_t s, uint32_t* out)
 {
     if (const char* v = std::getenv("IMIN_TIER0_VERTICES"); v && *v) {
@@ -619,30 +636,34 @@ int cutoff_for(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t 
             return IMIN_OK;
         }
     }
-    // A short call cannot repay the tuning: one of few samples, whose warm-up would tell nothing, or
-    // one that the warm-up shows to be shorter than the timed calls. It takes the default, which is
-    // within a few percent of the best, and the first longer call tunes. First call of theta = 256 on
-    // a 2,000-vertex graph 0.46 -> 0.21 ms; of AdvancedGreedy there (theta = 10^4, b = 10) 10.1 -> 2.1
-    // ms; of a batch of 48 new queries 467 -> 52 ms.
-    if (theta_hint > 0 && theta_hint < kTuneMinTheta) return IMIN_OK;
-    if (theta_hint > 0) {
+    // A short call cannot repay the tuning, which gives a few percent and costs about as much as the
+    // samples it times. So the samples of a graph's calls (all rounds of a greedy call) are added up,
+    // and the tuner runs when they come to kTuneRepay times the ones it would time; until then calls
+    // take the default. A program of many short calls is tuned like one of a single long call, and 50
+    // rounds of 25 ms tune at once.
+    // First call of theta = 256 on a 2,000-vertex graph 0.46 -> 0.21 ms; of AdvancedGreedy there
+    // (theta = 10^4, b = 10) 10.1 -> 2.1 ms; of a batch of 48 new queries 467 -> 52 ms.
+    uint64_t drawn = 0, need = 0;
+    {
         std::lock_guard<std::mutex> lk2(g_tune_mu);
-        const auto it = g_warm.find({g->fingerprint, cls});
-        if (it != g_warm.end() && theta_hint * it->second < kTuneMinCallMs) return IMIN_OK;
+        if (g_untuned.size() >= kUntunedMax) g_untuned.clear();  // only the counts start again
+        Untuned& u = g_untuned[{g->fingerprint, cls}];
+        u.samples += samples;
+        if (u.samples < u.need) return IMIN_OK;
+        drawn = u.samples;
     }
     int32_t best = -1;
-    float per_sample = 0.f;
-    const int rc = tune_cutoff(g, seeds, key, s, theta_hint, &best, &per_sample);
+    const int rc = tune_cutoff(g, seeds, key, s, drawn, &best, &need);
     if (rc) return rc;
+    std::lock_guard<std::mutex> lk2(g_tune_mu);
     if (best < 0) {
-        std::lock_guard<std::mutex> lk2(g_tune_mu);
-        g_warm[{g->fingerprint, cls}] = per_sample;
+        g_untuned[{g->fingerprint, cls}].need = need;
         return IMIN_OK;
     }
     *out = static_cast<uint32_t>(best);
-    g->cutoff[cls] = static_cast<int32_t>(*out);
-    std::lock_guard<std::mutex> lk2(g_tune_mu);
-    g_tuned[{g->fingerprint, cls}] = static_cast<int32_t>(*out);
+    g->cutoff[cls] = best;
+    g_tuned[{g->fingerprint, cls}] = best;
+    g_untuned.erase({g->fingerprint, cls});
     return IMIN_OK;
 }
 
@@ -650,10 +671,10 @@ int cutoff_for(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t 
 
 namespace imin {
 
-int tuned_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t key, uint32_t theta_hint,
+int tuned_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t key, uint64_t samples,
                  cudaStream_t s, uint32_t* out)
 {
-    return cutoff_for(g, seeds, key, theta_hint, s, out);
+    return cutoff_for(g, seeds, key, samples, s, out);
 }
 
 }  // namespace imin
@@ -844,7 +865,8 @@ int greedy_impl(Driver which, const imin_graph* g, const int32_t* seeds, int32_t
     if (b == 0) return IMIN_OK;
 
     uint32_t cutoff = 0;
-    rc = cutoff_for(g, hseeds, key, theta, s, &cutoff);
+    const int32_t rounds = std::min<int32_t>(b, g->n - n_seeds);
+    rc = cutoff_for(g, hseeds, key, static_cast<uint64_t>(theta) * rounds, s, &cutoff);
     if (rc) return rc;
     Query q(s);
     rc = setup_query(g, hseeds, theta, nullptr, cutoff, q);
@@ -1052,7 +1074,9 @@ int batch_impl(Driver which, imin_query* qs, int32_t nq, void* stream, uint32_t 
     for (int32_t i = 0; i < nq; ++i) {
         if (static_cast<uint32_t>(qs[i].n_seeds) > kBatchWarpMaxSeeds) continue;
         uint32_t c = 0;
-        const int rc = tuned_cutoff(qs[i].graph, hseeds[i], qs[i].key, qs[i].theta, s, &c);
+        const int32_t rounds = std::min<int32_t>(qs[i].b, qs[i].graph->n - qs[i].n_seeds);
+        const uint64_t samples = static_cast<uint64_t>(qs[i].theta) * rounds;
+        const int rc = tuned_cutoff(qs[i].graph, hseeds[i], qs[i].key, samples, s, &c);
         if (rc) return rc;
         if (c > 0) {
             warp_q[i] = 1;
@@ -1492,10 +1516,10 @@ int imin_autotune(const imin_graph* g, const int32_t* seeds, int32_t n_seeds, ui
     int rc = common_checks(g, seeds, n_seeds, 1, s, hseeds, mark);
     if (rc) return rc;
     int32_t c = 0;
-    float per_sample = 0.f;
+    uint64_t need = 0;
     {
         std::lock_guard<std::mutex> lk(g->tune_mu);
-        rc = tune_cutoff(g, hseeds, key, s, 0, &c, &per_sample);
+        rc = tune_cutoff(g, hseeds, key, s, 0, &c, &need);
         if (rc) return rc;
         g->cutoff[size_class(hseeds.size())] = c;
         std::lock_guard<std::mutex> lk2(g_tune_mu);

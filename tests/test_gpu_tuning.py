@@ -1,0 +1,96 @@
+"""When the warp/block cutoff is tuned: by the samples that the calls on a graph and seed-set size
+class draw together, over all their rounds. Launch counts tell a call that tuned from one that ran
+only its own kernels; results never depend on it."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2302_13529_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+TIMED_CALLS = 15  # 5 candidates, 3 calls each, of at least 2 kernels
+
+
+@pytest.fixture(autouse=True)
+def _tuner_on(monkeypatch):
+    monkeypatch.delenv("IMIN_TIER0_VERTICES", raising=False)
+    monkeypatch.delenv("IMIN_AUTOTUNE", raising=False)
+
+
+def _launches(lib, call):
+    c0 = lib.launch_count()
+    out = call()
+    return lib.launch_count() - c0, out
+
+
+def _chung_lu(n, m, seed):
+    rp, col = W.chung_lu(n, m, 2.1, seed)
+    return W.Graph(n, rp, col, W.wc_thresholds(col, n))
+
+
+def test_all_rounds_of_a_greedy_call_count(cuda_lib):
+    """71 rounds of 10^5 samples, each far shorter than the tuning, are more than 16 times the samples
+    it times (15 calls of at most 24 per resident block): the first call tunes."""
+    g = _chung_lu(2000, 10000, 501)
+    gh = cuda_lib.load_graph(g)
+    s = W.uniform_seeds(g.n, 10, 502)
+    first, b1 = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, 71, 100_000, 7))
+    second, b2 = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, 71, 100_000, 7))
+    third, b3 = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, 71, 100_000, 7))
+    assert first >= second + 2 * TIMED_CALLS and second == third, (first, second, third)
+    assert np.array_equal(b1, b2) and np.array_equal(b2, b3)
+
+
+def test_short_calls_add_up_and_a_long_one_tunes(cuda_lib):
+    """512 samples: default cutoff, own kernels only. The next 512 bring the sum to 1,024 and run the
+    warm-up, once. A batch query and a request count too, and the call that completes the sum tunes."""
+    g = _chung_lu(2000, 10000, 511)
+    gh = cuda_lib.load_graph(g)
+    s = W.uniform_seeds(g.n, 10, 512)
+    want = O.decrease(g, s, [], 512, 3, 0)
+    counts = []
+    for _ in range(4):
+        n, got = _launches(cuda_lib, lambda: cuda_lib.estimate_decrease(gh, s, [], 512, 3, 0))
+        assert np.array_equal(got, want)
+        counts.append(n)
+    assert counts[1] > counts[0] == counts[2] == counts[3], counts
+    cuda_lib.batch_advanced_greedy([(gh, s, 35, 100_000, 7)])
+    tuned, _ = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, 37, 100_000, 7))
+    after, _ = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, 37, 100_000, 7))
+    assert tuned >= after + 2 * TIMED_CALLS, (tuned, after)
+    assert np.array_equal(cuda_lib.estimate_decrease(gh, s, [], 512, 3, 0), want)
+
+
+def test_huge_cascades_drop_the_warp_tier_below_1024_samples_a_round(cuda_lib, monkeypatch):
+    """Three rounds of 600 samples on a graph whose cascades all outgrow the warp tier: the warm-up sees
+    it, and the rounds run without that tier, like calls with a forced cutoff of 0."""
+    rp, col = W.chung_lu(8000, 48000, 2.1, 521)
+    g = W.Graph(8000, rp, col, np.full(len(col), int(0.3 * 2**32), np.uint32))
+    gh = cuda_lib.load_graph(g)
+    hubs = np.argsort(-g.out_degree())[:20].astype(np.int32)
+    cuda_lib.advanced_greedy(gh, hubs, 3, 600, 7)
+    got, b = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, hubs, 3, 600, 7))
+    monkeypatch.setenv("IMIN_TIER0_VERTICES", "0")
+    forced, b0 = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, hubs, 3, 600, 7))
+    monkeypatch.setenv("IMIN_TIER0_VERTICES", "96")
+    with_warp, _ = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, hubs, 3, 600, 7))
+    assert got == forced < with_warp, (got, forced, with_warp)
+    assert np.array_equal(b, b0) and np.array_equal(b, O.advanced_greedy(g, hubs, 3, 600, 7))
+
+
+def test_a_tuned_cutoff_is_shared_by_handles_of_one_graph(cuda_lib):
+    """The first handle is tuned; a second one of the same graph takes its cutoff: the call that would
+    otherwise run the warm-up launches only its own kernels and fills the same tiers."""
+    g = W.graph_rmat_wc(12, 40000, seed=531)
+    s = W.uniform_seeds(g.n, 20, seed=532)
+    want = O.decrease(g, s, [], 2000, 43, 1)
+    h1 = cuda_lib.load_graph(g)
+    cuda_lib.autotune(h1, s, 43)
+    n1, (d1, st1) = _launches(cuda_lib, lambda: cuda_lib.estimate_decrease(h1, s, [], 2000, 43, 1, stats=True))
+    h2 = cuda_lib.load_graph(g)
+    n2, (d2, st2) = _launches(cuda_lib, lambda: cuda_lib.estimate_decrease(h2, s, [], 2000, 43, 1, stats=True))
+    assert n1 == n2 <= 4 and st1["tier_samples"] == st2["tier_samples"], (n1, n2, st1, st2)
+    assert np.array_equal(d1, want) and np.array_equal(d2, want)
