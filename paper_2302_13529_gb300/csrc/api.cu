@@ -297,6 +297,7 @@ int setup_query(const imin_graph* g, const std::vector<int32_t>& seeds, uint32_t
     cudaStream_t s = q.arena.s;
     q.words = (g->n + 31) / 32;
     q.plan = plan_tiers(g->dev, g->n, g->m, static_cast<uint32_t>(seeds.size()), cutoff);
+    q.plan.few = few_per_warp(q.plan, theta);
     std::vector<int32_t>& ids = q.ids;
     ids = seeds;
     if (blocked != nullptr) ids.insert(ids.end(), blocked->begin(), blocked->end());
@@ -512,14 +513,16 @@ int size_class(size_t ns)
     return c;
 }
 
-// Device time of one Alg. 2 call (round 0, no blockers) with the given cutoff.
+// Device time of one Alg. 2 call (round 0, no blockers) of `theta` samples with the given cutoff, on the
+// kernels of a call of `as_theta` samples.
 // warp_done (optional): receives the number of samples the warp tier 0 finished.
 int time_call(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t key, uint32_t cutoff,
-              uint32_t theta, cudaStream_t s, float* ms, unsigned long long* warp_done = nullptr)
+              uint32_t theta, uint32_t as_theta, cudaStream_t s, float* ms, unsigned long long* warp_done = nullptr)
 {
     Query q(s);
     int rc = setup_query(g, seeds, theta, nullptr, cutoff, q);
     if (rc) return rc;
+    q.plan.few = few_per_warp(q.plan, as_theta);
     RoundCtl* const ctl = q.ctl;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     IMIN_CUDA(cudaEventCreate(&e0));
@@ -547,22 +550,23 @@ int time_call(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t k
     return check_ctl(hctl);
 }
 
+// as_theta: samples per round of the call the tuning is for, whose kernels are timed.
 // drawn: samples that the calls so far have drawn on this graph (0: tune in any case). *out < 0: they
 // have not earned the tuning yet (its timed calls are more than a kTuneRepay-th of them); no candidate
 // was timed, and *need is the number of samples that will.
 int tune_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t key, cudaStream_t s,
-                uint64_t drawn, int32_t* out, uint64_t* need)
+                uint32_t as_theta, uint64_t drawn, int32_t* out, uint64_t* need)
 {
     constexpr int kCand = static_cast<int>(sizeof(kCutoffs) / sizeof(kCutoffs[0]));
     float warm = 0.f, t[kCand];
     const uint32_t blocks = cta_blocks(g, seeds.size());
     const uint32_t tw = kTuneWarmup;
     unsigned long long warp_done = 0;
-    int rc = time_call(g, seeds, key, kDefaultCutoff, tw, s, &warm, &warp_done);  // warm-up, cost
+    int rc = time_call(g, seeds, key, kDefaultCutoff, tw, as_theta, s, &warm, &warp_done);  // warm-up, cost
     if (rc) return rc;
     const auto costly = [&] { return kTuneCallMs * tw < 4.0 * blocks * warm; };
     if (costly()) {  // once more: a process's first call also waits for its kernels to be loaded
-        rc = time_call(g, seeds, key, kDefaultCutoff, tw, s, &warm, &warp_done);
+        rc = time_call(g, seeds, key, kDefaultCutoff, tw, as_theta, s, &warm, &warp_done);
         if (rc) return rc;
     }
     double per_sample = std::max(1e-7, static_cast<double>(warm) / tw);  // ms
@@ -581,7 +585,7 @@ int tune_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t
     // samples it makes room for; re-estimate on a call of that size
     uint32_t theta = static_cast<uint32_t>(std::min<double>({kTuneCallMs / per_sample, 24.0 * blocks, 65536.0}));
     if (too_early(theta)) return IMIN_OK;
-    rc = time_call(g, seeds, key, kDefaultCutoff, theta, s, &warm);
+    rc = time_call(g, seeds, key, kDefaultCutoff, theta, as_theta, s, &warm);
     if (rc) return rc;
     per_sample = std::max(1e-7, static_cast<double>(warm) / theta);
     theta = static_cast<uint32_t>(std::min<double>({std::max(kTuneCallMs / per_sample, 4.0 * blocks),
@@ -590,7 +594,7 @@ int tune_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t
     for (int rep = 0; rep < kTuneReps; ++rep) {
         for (int i = 0; i < kCand; ++i) {
             float ms = 0.f;
-            rc = time_call(g, seeds, key, kCutoffs[i], theta, s, &ms);
+            rc = time_call(g, seeds, key, kCutoffs[i], theta, as_theta, s, &ms);
             if (rc) return rc;
             t[i] = rep == 0 ? ms : std::min(t[i], ms);
         }
@@ -604,9 +608,9 @@ int tune_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t
 
 // The cutoff for a call: IMIN_TIER0_VERTICES forces one; IMIN_AUTOTUNE=0, or a stream being
 // captured (the tuner synchronizes), gives the default; otherwise the tuned value, tuning on first
-// use for this graph and seed-set size class, once its calls have drawn enough samples. samples: what
-// this call draws over all its rounds.
-int cutoff_for(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t key, uint64_t samples,
+// use for this graph and seed-set size class, once its calls have drawn enough samples. rounds, theta:
+// of this call.
+int cutoff_for(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t key, uint32_t theta, int32_t rounds,
                cudaStream_t s, uint32_t* out)
 {
     if (const char* v = std::getenv("IMIN_TIER0_VERTICES"); v && *v) {
@@ -648,12 +652,12 @@ int cutoff_for(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t 
         std::lock_guard<std::mutex> lk2(g_tune_mu);
         if (g_untuned.size() >= kUntunedMax) g_untuned.clear();  // only the counts start again
         Untuned& u = g_untuned[{g->fingerprint, cls}];
-        u.samples += samples;
+        u.samples += static_cast<uint64_t>(theta) * rounds;
         if (u.samples < u.need) return IMIN_OK;
         drawn = u.samples;
     }
     int32_t best = -1;
-    const int rc = tune_cutoff(g, seeds, key, s, drawn, &best, &need);
+    const int rc = tune_cutoff(g, seeds, key, s, theta, drawn, &best, &need);
     if (rc) return rc;
     std::lock_guard<std::mutex> lk2(g_tune_mu);
     if (best < 0) {
@@ -671,10 +675,10 @@ int cutoff_for(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t 
 
 namespace imin {
 
-int tuned_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t key, uint64_t samples,
-                 cudaStream_t s, uint32_t* out)
+int tuned_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t key, uint32_t theta,
+                 int32_t rounds, cudaStream_t s, uint32_t* out)
 {
-    return cutoff_for(g, seeds, key, samples, s, out);
+    return cutoff_for(g, seeds, key, theta, rounds, s, out);
 }
 
 }  // namespace imin
@@ -699,7 +703,7 @@ int estimate_impl(const imin_graph* g, const int32_t* seeds, int32_t n_seeds,
 
     const bool dev_out = is_device_ptr(out_delta);
     uint32_t cutoff = 0;
-    rc = cutoff_for(g, hseeds, key, theta, s, &cutoff);
+    rc = cutoff_for(g, hseeds, key, theta, 1, s, &cutoff);
     if (rc) return rc;
     Query q(s);
     rc = setup_query(g, hseeds, theta, dev_out ? reinterpret_cast<unsigned long long*>(out_delta) : nullptr,
@@ -866,7 +870,7 @@ int greedy_impl(Driver which, const imin_graph* g, const int32_t* seeds, int32_t
 
     uint32_t cutoff = 0;
     const int32_t rounds = std::min<int32_t>(b, g->n - n_seeds);
-    rc = cutoff_for(g, hseeds, key, static_cast<uint64_t>(theta) * rounds, s, &cutoff);
+    rc = cutoff_for(g, hseeds, key, theta, rounds, s, &cutoff);
     if (rc) return rc;
     Query q(s);
     rc = setup_query(g, hseeds, theta, nullptr, cutoff, q);
@@ -1075,8 +1079,7 @@ int batch_impl(Driver which, imin_query* qs, int32_t nq, void* stream, uint32_t 
         if (static_cast<uint32_t>(qs[i].n_seeds) > kBatchWarpMaxSeeds) continue;
         uint32_t c = 0;
         const int32_t rounds = std::min<int32_t>(qs[i].b, qs[i].graph->n - qs[i].n_seeds);
-        const uint64_t samples = static_cast<uint64_t>(qs[i].theta) * rounds;
-        const int rc = tuned_cutoff(qs[i].graph, hseeds[i], qs[i].key, samples, s, &c);
+        const int rc = tuned_cutoff(qs[i].graph, hseeds[i], qs[i].key, qs[i].theta, rounds, s, &c);
         if (rc) return rc;
         if (c > 0) {
             warp_q[i] = 1;
@@ -1519,7 +1522,7 @@ int imin_autotune(const imin_graph* g, const int32_t* seeds, int32_t n_seeds, ui
     uint64_t need = 0;
     {
         std::lock_guard<std::mutex> lk(g->tune_mu);
-        rc = tune_cutoff(g, hseeds, key, s, 0, &c, &need);
+        rc = tune_cutoff(g, hseeds, key, s, UINT32_MAX, 0, &c, &need);
         if (rc) return rc;
         g->cutoff[size_class(hseeds.size())] = c;
         std::lock_guard<std::mutex> lk2(g_tune_mu);

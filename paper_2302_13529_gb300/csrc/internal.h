@@ -72,6 +72,7 @@ struct TierPlan {
     uint64_t smem_bytes[kTiers];  // dynamic shared memory per block
     uint64_t scratch_bytes[kTiers];
     bool use_cta = false;         // tier 3 replaces tiers 0 and 1
+    bool few = false;             // tier 0 with the register budget for few samples per warp
     CtaCfg cta{};
 };
 
@@ -84,6 +85,8 @@ void tier0_cfg(uint32_t ns, uint32_t r0, TierCfg* c);
 // fit). allow_tier0_smem must have run once on the device.
 void plan_tier0(const DeviceInfo& dev, uint32_t ns, uint32_t cutoff, TierPlan* p);
 void allow_tier0_smem(const DeviceInfo& dev);
+// Whether a call of theta samples per round is one of few samples per warp of the plan's tier 0.
+bool few_per_warp(const TierPlan& p, uint32_t theta);
 // cutoff: non-seed capacity of the warp tier 0 run in front of the block tier (0: none).
 TierPlan plan_tiers(const DeviceInfo& dev, int32_t n, int32_t m, uint32_t ns, uint32_t cutoff);
 
@@ -141,10 +144,10 @@ cudaError_t launch_batch_warp(const BatchStep& B, const TierCfg& c, uint32_t blo
                               cudaStream_t s);
 // The warp/block cutoff of one query (api.cu): IMIN_TIER0_VERTICES when set; kDefaultCutoff with
 // IMIN_AUTOTUNE=0 or on a capturing stream; otherwise the autotuner's value for the graph and the
-// seed-set size class, tuned on `s` and cached once the calls on them, this one of `samples` samples
-// included, have drawn enough to repay it (kDefaultCutoff until then).
-int tuned_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t key, uint64_t samples,
-                 cudaStream_t s, uint32_t* out);
+// seed-set size class, tuned on `s` and cached once the calls on them, this one of `rounds` rounds of
+// theta samples included, have drawn enough to repay it (kDefaultCutoff until then).
+int tuned_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t key, uint32_t theta,
+                 int32_t rounds, cudaStream_t s, uint32_t* out);
 
 // Selection (Alg. 3/4 argmax) -----------------------------------------------------------------
 struct SelectParams {

@@ -238,7 +238,10 @@ extern "C" int imin_estimate_decrease_noalloc(const imin_graph* g, const int32_t
     // against 0.23.
     const bool whole_only = theta <= (small.rcap < cfg.rcap ? 20u : 4u) * whole_blocks;
     TierPlan warp{};
-    if (!whole_only) plan_tier0(g->dev, static_cast<uint32_t>(n_seeds), kDefaultCutoff, &warp);
+    if (!whole_only) {
+        plan_tier0(g->dev, static_cast<uint32_t>(n_seeds), kDefaultCutoff, &warp);
+        warp.few = few_per_warp(warp, theta);
+    }
 
     RoundCtl* ctl = reinterpret_cast<RoundCtl*>(base + off_ctl);
     uint32_t* bad = reinterpret_cast<uint32_t*>(base + off_bad);

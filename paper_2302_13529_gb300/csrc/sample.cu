@@ -178,6 +178,11 @@ void allow_tier0_smem(const DeviceInfo& dev)
     allow_max_dynamic_smem(k_sample_tier<0, kModelIC, kFewPerSm>, dev);
 }
 
+bool few_per_warp(const TierPlan& p, uint32_t theta)
+{
+    return theta <= kFewPerWarp * kWarpsPerBlock * p.blocks[0];
+}
+
 void plan_tier0(const DeviceInfo& dev, uint32_t ns, uint32_t cutoff, TierPlan* p)
 {
     tier0_cfg(ns, cutoff, &p->cfg[0]);
@@ -284,7 +289,7 @@ cudaError_t launch_sample_tier(int tier, const SampleParams& P, const TierPlan& 
     // the first tier that runs takes the whole sample range; tier 0 is skipped only when the
     // seed set does not fit its shared-memory working set
     c.from_range = tier == 0 || (tier == 1 && plan.blocks[0] == 0 && !plan.use_cta);
-    const bool few = tier == 0 && P.theta <= kFewPerWarp * kWarpsPerBlock * plan.blocks[0];
+    const bool few = tier == 0 && plan.few;
     const dim3 grid(plan.blocks[tier]), block(kWarpsPerBlock * 32);
     const size_t sm = plan.smem_bytes[tier];
     if (P.g.lo4 == nullptr) {

@@ -313,9 +313,8 @@ void imin_server::run()
         bool need_cb = false;
         for (Req* r : admitted) {
             if (r->warp) {
-                const uint64_t samples =
-                    static_cast<uint64_t>(r->theta) * std::min<int32_t>(r->b, r->g->n - static_cast<int32_t>(r->seeds.size()));
-                const int rc = tuned_cutoff(r->g, r->seeds, r->key, samples, s, &r->cutoff);
+                const int32_t rounds = std::min<int32_t>(r->b, r->g->n - static_cast<int32_t>(r->seeds.size()));
+                const int rc = tuned_cutoff(r->g, r->seeds, r->key, r->theta, rounds, s, &r->cutoff);
                 if (rc != IMIN_OK) {
                     fail_all(rc, "warp/block cutoff tuning failed");
                     return;

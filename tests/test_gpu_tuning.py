@@ -94,3 +94,31 @@ def test_a_tuned_cutoff_is_shared_by_handles_of_one_graph(cuda_lib):
     n2, (d2, st2) = _launches(cuda_lib, lambda: cuda_lib.estimate_decrease(h2, s, [], 2000, 43, 1, stats=True))
     assert n1 == n2 <= 4 and st1["tier_samples"] == st2["tier_samples"], (n1, n2, st1, st2)
     assert np.array_equal(d1, want) and np.array_equal(d2, want)
+
+
+@pytest.mark.parametrize("theta,rounds,budget", [(100_000, 71, 5), (7_000, 1001, 4)])
+def test_the_tuner_times_the_kernels_of_the_call(cuda_lib, theta, rounds, budget):
+    """The warp tier has one instantiation for rounds of more than two samples per resident warp (5 blocks
+    per SM) and one for fewer (4); the line lies at 7,296 samples where a cutoff leaves 3 blocks per SM,
+    at 12,160 where it leaves 5. A call that tunes runs only its own, in the timed calls too, whose
+    sample counts lie on both sides of that line."""
+    import re
+
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+
+    g = _chung_lu(2000, 10000, 541 + budget)
+    gh = cuda_lib.load_graph(g)
+    s = W.uniform_seeds(g.n, 10, 542)
+    with profile(activities=[ProfilerActivity.CUDA]):  # the first use sets the profiler up
+        torch.zeros(1, device="cuda")
+        torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        n, _ = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, rounds, theta, 7))
+        torch.cuda.synchronize()
+    own, _ = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, rounds, theta, 7))
+    assert n >= own + 2 * TIMED_CALLS, (n, own)
+    seen = [m.group(1) for e in prof.events() if (m := re.search(r"k_sample_tier<0, 0, (\d)u?>", e.name))]
+    if not seen:
+        pytest.skip("no kernel records from the profiler here")
+    assert set(seen) == {str(budget)} and len(seen) > TIMED_CALLS, (set(seen), len(seen))
