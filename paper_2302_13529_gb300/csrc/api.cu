@@ -287,12 +287,13 @@ struct CallStatus {
 };
 static_assert(offsetof(CallStatus, stats) == kStatsOffset, "as setup_query lays them out");
 
-// blocked: vertices masked with the seeds (NULL: none). A small call is bound by what the host
+// blocked: vertices masked with the seeds (NULL: none). spread: a call of the spread kernels, which have
+// no counters, sample lists or whole-graph slots (1 GiB). A small call is bound by what the host
 // enqueues, so its small buffers come in one allocation with one clear, and all its ids in one copy
 // and one mask kernel (theta = 256 on a 2,000-vertex graph: 0.152 -> 0.134 ms).
 int setup_query(const imin_graph* g, const std::vector<int32_t>& seeds, uint32_t theta,
                 unsigned long long* out_delta_dev, uint32_t cutoff, Query& q,
-                const std::vector<int32_t>* blocked = nullptr)
+                const std::vector<int32_t>* blocked = nullptr, bool spread = false)
 {
     cudaStream_t s = q.arena.s;
     q.words = (g->n + 31) / 32;
@@ -311,12 +312,14 @@ int setup_query(const imin_graph* g, const std::vector<int32_t>& seeds, uint32_t
     q.seeds = reinterpret_cast<int32_t*>(small + off_ids);
     if (out_delta_dev != nullptr) {
         q.delta = out_delta_dev;
-    } else {
+    } else if (!spread) {
         IMIN_CUDA(q.arena.alloc(&q.delta, g->n));
     }
-    IMIN_CUDA(q.arena.alloc(&q.lists, static_cast<uint64_t>(kTiers) * theta));
-    if (q.plan.scratch_bytes[1] > 0) IMIN_CUDA(q.arena.alloc(&q.scratch1, q.plan.scratch_bytes[1]));
-    IMIN_CUDA(q.arena.alloc(&q.scratch2, q.plan.scratch_bytes[2]));
+    if (!spread) {
+        IMIN_CUDA(q.arena.alloc(&q.lists, static_cast<uint64_t>(kTiers) * theta));
+        if (q.plan.scratch_bytes[1] > 0) IMIN_CUDA(q.arena.alloc(&q.scratch1, q.plan.scratch_bytes[1]));
+        IMIN_CUDA(q.arena.alloc(&q.scratch2, q.plan.scratch_bytes[2]));
+    }
     // with the warp tier in front of the block tier, one hand-off snapshot per sample it may give
     // up on, after the block tier's slots: the block tier resumes those samples where it stopped
     uint64_t handoff_bytes = 0;
@@ -330,9 +333,11 @@ int setup_query(const imin_graph* g, const std::vector<int32_t>& seeds, uint32_t
     if (q.plan.use_cta) IMIN_CUDA(prepare_cta_scratch(q.plan.cta, q.plan.blocks[kTierCta], q.scratch3, s));
     IMIN_CUDA(cudaMemcpyAsync(q.seeds, ids.data(), sizeof(int32_t) * ids.size(), cudaMemcpyHostToDevice, s));
     IMIN_CUDA(cudaMemsetAsync(small, 0, off_ids, s));
-    IMIN_CUDA(cudaMemsetAsync(q.delta, 0, sizeof(unsigned long long) * g->n, s));
-    IMIN_CUDA(prepare_warp_slots(q.plan, 1, q.scratch1, s));
-    IMIN_CUDA(prepare_warp_slots(q.plan, kTierWhole, q.scratch2, s));
+    if (!spread) {
+        IMIN_CUDA(cudaMemsetAsync(q.delta, 0, sizeof(unsigned long long) * g->n, s));
+        IMIN_CUDA(prepare_warp_slots(q.plan, 1, q.scratch1, s));
+        IMIN_CUDA(prepare_warp_slots(q.plan, kTierWhole, q.scratch2, s));
+    }
     IMIN_CUDA(launch_build_excl(q.excl, q.seeds, static_cast<int32_t>(ids.size()), s));
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return IMIN_OK;
@@ -358,20 +363,36 @@ cudaError_t enqueue_call(const SampleParams& P, const Query& q, CallTimer& T)
     return cudaSuccess;
 }
 
-// All slices of a spread call (spread.cu): the warp kernel and the block kernel of each.
-cudaError_t enqueue_spread(const SampleParams& P, const Query& q, CallTimer& T, const int32_t* sets, uint32_t k,
-                           unsigned long long items, uint32_t* handoff, unsigned long long* sums)
+// All slices of a spread call (spread.cu): the warp kernel and the block kernel of each. The slices
+// get shorter until their hand-offs (1 KB per item) fit the device's free memory: a call that needs few
+// slots must not fail for a buffer that only saves launches. IMIN_SPREAD_HANDOFF_MIB lowers the limit,
+// for tests.
+cudaError_t enqueue_spread(const SampleParams& P, Query& q, CallTimer& T, const int32_t* sets, uint32_t k,
+                           unsigned long long items, unsigned long long* sums)
 {
-    for (unsigned long long i = 0; i < spread_slices(items); ++i) {
-        const cudaError_t e = T.run(kKindCta, [&](bool* launched) {
+    constexpr unsigned long long kShortest = 1024;
+    unsigned long long slice = std::min(items, kSpreadSlice);
+    if (const char* v = std::getenv("IMIN_SPREAD_HANDOFF_MIB"); v && *v) {
+        const unsigned long long room = std::strtoull(v, nullptr, 10) << 20;
+        slice = std::min(slice, std::max(1ull, room / (4 * spread_handoff_words(1))));
+    }
+    uint32_t* handoff = nullptr;
+    cudaError_t e = q.arena.alloc(&handoff, spread_handoff_words(slice));
+    while (e == cudaErrorMemoryAllocation && slice > kShortest) {
+        cudaGetLastError();
+        slice /= 2;
+        e = q.arena.alloc(&handoff, spread_handoff_words(slice));
+    }
+    if (e == cudaSuccess) e = prepare_spread(q.plan.cta);
+    for (unsigned long long i = 0; i < items && e == cudaSuccess; i += slice) {
+        e = T.run(kKindCta, [&](bool* launched) {
             *launched = true;
             g_launches.fetch_add(1, std::memory_order_relaxed);  // the slice's second kernel
             return launch_spread_slice(P, q.plan.cta, q.plan.blocks[kTierCta], q.plan.smem_bytes[kTierCta],
-                                       q.scratch3, sets, k, items, i, handoff, sums, T.s);
+                                       q.scratch3, sets, k, i, std::min(items, i + slice), handoff, sums, T.s);
         });
-        if (e != cudaSuccess) return e;
     }
-    return cudaSuccess;
+    return e;
 }
 
 cudaError_t enqueue_select(const SelectParams& sp, CallTimer& T)
@@ -745,17 +766,15 @@ int spread_impl(const imin_graph* g, const int32_t* seeds, int32_t n_seeds, cons
     if (rc) return rc;
 
     Query q(s);
-    rc = setup_query(g, hseeds, theta, nullptr, 0, q, &hblocked);
+    rc = setup_query(g, hseeds, theta, nullptr, 0, q, &hblocked, true);
     if (rc) return rc;
     if (!q.plan.use_cta) return fail(IMIN_ERR_INTERNAL, "the spread kernel needs the block-per-sample tier");
     unsigned long long* dsum = nullptr;
-    uint32_t* handoff = nullptr;
-    IMIN_CUDA(q.arena.alloc(&handoff, spread_handoff_words(theta)));
     IMIN_CUDA(q.arena.alloc(&dsum, 1));
     IMIN_CUDA(cudaMemsetAsync(dsum, 0, sizeof(unsigned long long), s));
     CallTimer T(s);
     const SampleParams P = sample_params(g, q, static_cast<uint32_t>(n_seeds), theta, key, round, q.ctl, nullptr);
-    IMIN_CUDA(enqueue_spread(P, q, T, nullptr, 0, theta, handoff, dsum));
+    IMIN_CUDA(enqueue_spread(P, q, T, nullptr, 0, theta, dsum));
     CallStatus status;
     unsigned long long hsum = 0;
     IMIN_CUDA(cudaMemcpyAsync(&status, q.ctl, sizeof(status), cudaMemcpyDeviceToHost, s));
@@ -800,23 +819,21 @@ int spread_sets_core(const imin_graph* g, const std::vector<int32_t>& hseeds, co
         if (rc) return rc;
     }
     Query q(s);
-    int rc = setup_query(g, hseeds, theta, nullptr, 0, q, &hblocked);
+    int rc = setup_query(g, hseeds, theta, nullptr, 0, q, &hblocked, true);
     if (rc) return rc;
     if (!q.plan.use_cta) return fail(IMIN_ERR_INTERNAL, "the spread kernel needs the block-per-sample tier");
     int32_t* dsets = nullptr;
     unsigned long long* dsums = nullptr;
-    uint32_t* handoff = nullptr;
     const unsigned long long items = static_cast<unsigned long long>(nsets) * theta;
     IMIN_CUDA(q.arena.alloc(&dsets, static_cast<uint64_t>(nsets) * k));
     IMIN_CUDA(q.arena.alloc(&dsums, static_cast<uint64_t>(nsets)));
-    IMIN_CUDA(q.arena.alloc(&handoff, spread_handoff_words(items)));
     IMIN_CUDA(cudaMemsetAsync(dsums, 0, sizeof(unsigned long long) * nsets, s));
     if (k > 0)
         IMIN_CUDA(cudaMemcpyAsync(dsets, hsets, sizeof(int32_t) * nsets * k, cudaMemcpyHostToDevice, s));
     CallTimer T(s);
     SampleParams P = sample_params(g, q, static_cast<uint32_t>(hseeds.size()), theta, key, round, q.ctl, nullptr);
     P.stats = nullptr;
-    IMIN_CUDA(enqueue_spread(P, q, T, dsets, static_cast<uint32_t>(k), items, handoff, dsums));
+    IMIN_CUDA(enqueue_spread(P, q, T, dsets, static_cast<uint32_t>(k), items, dsums));
     RoundCtl hctl;
     IMIN_CUDA(cudaMemcpyAsync(&hctl, q.ctl, sizeof(hctl), cudaMemcpyDeviceToHost, s));
     IMIN_CUDA(cudaMemcpyAsync(hsums, dsums, sizeof(uint64_t) * nsets, cudaMemcpyDeviceToHost, s));

@@ -114,14 +114,16 @@ cudaError_t prepare_cta_scratch(const CtaCfg& c, uint32_t blocks, uint8_t* scrat
 
 // Monte-Carlo spread (spread.cu) over items of (blocker set, sample): item i adds |R| (seeds
 // included) of sample i % P.theta, with set i / P.theta (k vertices of `sets`) blocked on top of
-// P.excl, to sums[i / P.theta]. A call enqueues slices 0 .. spread_slices(items) - 1 in order, with
-// the block tier's layout `c` and `blocks` slots of `scratch` and with spread_handoff_words(items)
-// words of `handoff` (shared by the slices). P.ctl->error must start at 0.
-unsigned long long spread_slices(unsigned long long items);
+// P.excl, to sums[i / P.theta]. A call enqueues its items in slices [first, last) of at most
+// kSpreadSlice, in order, with the block tier's layout `c` and `blocks` slots of `scratch` and with
+// spread_handoff_words(last - first) words of `handoff` (shared by the slices). P.ctl->error must start
+// at 0. P needs no counters, lists or stats.
+constexpr unsigned long long kSpreadSlice = 1ull << 18;
 uint64_t spread_handoff_words(unsigned long long items);
+cudaError_t prepare_spread(const CtaCfg& c);  // once per call, before the first slice
 cudaError_t launch_spread_slice(const SampleParams& P, const CtaCfg& c, uint32_t blocks, uint64_t smem,
-                                uint8_t* scratch, const int32_t* sets, uint32_t k, unsigned long long items,
-                                unsigned long long slice, uint32_t* handoff, unsigned long long* sums,
+                                uint8_t* scratch, const int32_t* sets, uint32_t k, unsigned long long first,
+                                unsigned long long last, uint32_t* handoff, unsigned long long* sums,
                                 cudaStream_t s);
 
 // Batched multi-query steps (batch.cu).

@@ -38,8 +38,6 @@ constexpr uint32_t kSlots = 512;
 constexpr uint32_t kSlotShift = 23;    // 32 - log2(kSlots)
 constexpr uint32_t kHeader = 8;        // words before the queue in a hand-off
 constexpr uint32_t kHandoffWords = kHeader + kQueue;
-// Items per slice: bounds the hand-offs, one per item at most (277 MB).
-constexpr unsigned long long kSlice = 1ull << 18;
 
 // Items [first, last) of a call: item i is set i / theta, sample i % theta.
 struct SpreadWork {
@@ -321,35 +319,35 @@ cudaError_t launch_slice(const SampleParams& P, const CtaCfg& cfg, uint32_t warp
 
 }  // namespace
 
-uint64_t spread_handoff_words(unsigned long long items) { return std::min(items, kSlice) * kHandoffWords; }
+// One hand-off per item at most: 277 MB for a whole kSpreadSlice.
+uint64_t spread_handoff_words(unsigned long long items) { return items * kHandoffWords; }
 
-unsigned long long spread_slices(unsigned long long items) { return (items + kSlice - 1) / kSlice; }
+cudaError_t prepare_spread(const CtaCfg& c)
+{
+    const DeviceInfo dev = device_info();
+    const cudaError_t e = c.global_bitmap ? allow_max_dynamic_smem(k_spread_block<false, kModelIC>, dev)
+                                          : allow_max_dynamic_smem(k_spread_block<true, kModelIC>, dev);
+    if (e != cudaSuccess) return e;
+    return c.global_bitmap ? allow_max_dynamic_smem(k_spread_block<false, kModelLT>, dev)
+                           : allow_max_dynamic_smem(k_spread_block<true, kModelLT>, dev);
+}
 
 cudaError_t launch_spread_slice(const SampleParams& P, const CtaCfg& c, uint32_t blocks, uint64_t smem,
-                                uint8_t* scratch, const int32_t* sets, uint32_t k, unsigned long long items,
-                                unsigned long long slice, uint32_t* handoff, unsigned long long* sums,
+                                uint8_t* scratch, const int32_t* sets, uint32_t k, unsigned long long first,
+                                unsigned long long last, uint32_t* handoff, unsigned long long* sums,
                                 cudaStream_t s)
 {
     const DeviceInfo dev = device_info();
     CtaCfg cfg = c;
     cfg.scratch = scratch;
-    if (slice == 0) {
-        if (c.global_bitmap) {
-            allow_max_dynamic_smem(k_spread_block<false, kModelIC>, dev);
-            allow_max_dynamic_smem(k_spread_block<false, kModelLT>, dev);
-        } else {
-            allow_max_dynamic_smem(k_spread_block<true, kModelIC>, dev);
-            allow_max_dynamic_smem(k_spread_block<true, kModelLT>, dev);
-        }
-    }
     // the slice's work cursors and hand-off count (the error bits stay)
     const cudaError_t e = cudaMemsetAsync(P.ctl, 0, offsetof(RoundCtl, error), s);
     if (e != cudaSuccess) return e;
     SpreadWork W{};
     W.sets = sets;
     W.k = k;
-    W.first = kSlice * slice;
-    W.last = std::min(items, W.first + kSlice);
+    W.first = first;
+    W.last = last;
     const uint32_t n = static_cast<uint32_t>(W.last - W.first);
     const uint32_t warp_blocks = std::min((n + kWarps - 1) / kWarps, 5u * dev.sms);
     // at least 8 grabs per warp, so that no warp is left with the last long run

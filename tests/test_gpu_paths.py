@@ -193,3 +193,47 @@ def test_non_tree_edges_of_a_hand_off_against_the_slot_capacity(cuda_lib, monkey
     assert sum(st["tier_samples"]) == 3000 and st["tier_samples"][2] > 0
     want = O.advanced_greedy(g, s, 2, 500, 3)
     assert np.array_equal(cuda_lib.batch_advanced_greedy([(gh, s, 2, 500, 3)])[0], want)
+
+
+def _pool_high():
+    """Highest number of bytes in use in the device's default memory pool since the last call."""
+    import ctypes
+
+    cu = ctypes.CDLL("libcuda.so.1")
+    pool, high, zero = ctypes.c_void_p(), ctypes.c_uint64(), ctypes.c_uint64(0)
+    used_mem_high = 8  # CU_MEMPOOL_ATTR_USED_MEM_HIGH
+    assert cu.cuDeviceGetDefaultMemPool(ctypes.byref(pool), 0) == 0
+    assert cu.cuMemPoolGetAttribute(pool, used_mem_high, ctypes.byref(high)) == 0
+    assert cu.cuMemPoolSetAttribute(pool, used_mem_high, ctypes.byref(zero)) == 0  # down to what is in use
+    return high.value
+
+
+def test_spread_holds_only_what_it_uses(cuda_lib, monkeypatch):
+    """The spread kernels have no whole-graph slots (1 GiB at this size), sample lists or counters: beside
+    the block tier's slots, which an Alg. 2 call has too, a spread call holds its hand-offs, 1 KB a sample."""
+    rp, col = W.chung_lu(20_000, 100_000, 2.1, 61)
+    g = W.Graph(20_000, rp, col, W.wc_thresholds(col, 20_000))
+    gh = cuda_lib.load_graph(g)
+    monkeypatch.setenv("IMIN_TIER0_VERTICES", "0")
+    _pool_high()
+    cuda_lib.estimate_decrease(gh, [0, 1], [], 4000, 3, 0)
+    alg2 = _pool_high()
+    for call in (lambda: cuda_lib.estimate_spread(gh, [0, 1], [], 4000, 3, 0),
+                 lambda: cuda_lib.estimate_spread_sets(gh, [0, 1], [], [[5]], 4000, 3, 0)):
+        call()
+        assert _pool_high() < alg2 - 900_000_000
+
+
+@pytest.mark.parametrize("mib", [None, "1", "3"])
+def test_spread_in_slices(cuda_lib, monkeypatch, mib):
+    """More items than a slice holds (2^18, or what a lowered hand-off limit leaves: 992 and 2,978), with
+    a last slice that is not full and cascades on both routes."""
+    if mib is not None:
+        monkeypatch.setenv("IMIN_SPREAD_HANDOFF_MIB", mib)
+    g = _star(300, 0.87)  # 261 of 300 leaves on average, the queue holds 256
+    gh = cuda_lib.load_graph(g)
+    theta = 90_001 if mib is None else 2_001
+    sets = [[5], [6], [301]]
+    want = O.spread_sets(g, [0], [], sets, theta, 4, 1)
+    assert np.array_equal(cuda_lib.estimate_spread_sets(gh, [0], [], sets, theta, 4, 1), want)
+    assert cuda_lib.estimate_spread(gh, [0], [5], theta, 4, 1) == int(want[0])
