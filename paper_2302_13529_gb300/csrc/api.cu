@@ -696,6 +696,8 @@ int cutoff_for(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t 
 
 namespace imin {
 
+void count_launches(uint64_t kernels) { g_launches.fetch_add(kernels, std::memory_order_relaxed); }
+
 int tuned_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t key, uint32_t theta,
                  int32_t rounds, cudaStream_t s, uint32_t* out)
 {

@@ -32,6 +32,9 @@ cudaError_t allow_max_dynamic_smem(F func, const DeviceInfo& dev)
     return cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, avail > 0 ? avail : 0);
 }
 
+// Adds to imin_launch_count (kernels launched outside api.cu).
+void count_launches(uint64_t kernels);
+
 // Record `msg` as the calling thread's last error (fixed buffer, no allocation); returns code.
 int fail_msg(int code, const char* msg);
 

@@ -8,10 +8,11 @@
 // its kernel runs and the kernel's status after it, so it returns only when the counters are
 // final, and it cannot be recorded into a CUDA graph by stream capture.
 //
-// What it does: exactly what imin_estimate_decrease computes, with the warp tier at a fixed cutoff
-// (sample.cu) in front of the block-per-sample tier (sample_cta.cu), but every byte of working
-// memory it needs besides the caller's inputs and output comes from one file-scope device array of kNoAllocBytes (64 MiB). Every GPU that loads
-// the library holds that array until the process exits. Its limits follow from its size:
+// What it does: exactly what imin_estimate_decrease computes, with the block-per-sample tier
+// (sample_cta.cu) and, for many samples, the warp tier at a fixed cutoff (sample.cu) in front of it.
+// But every byte of working memory it needs besides the caller's inputs and output comes from one
+// file-scope device array of kNoAllocBytes (64 MiB). Every GPU that loads the library holds that
+// array until the process exits. Its limits follow from its size:
 // graphs with at most kNoAllocMaxVertices vertices and at most kNoAllocMaxTheta samples per call;
 // bigger requests are rejected with IMIN_ERR_INVALID. A sampled cascade that would need the
 // whole-graph fallback tier (more non-tree live edges or BFS levels than the block tier holds)
@@ -230,13 +231,20 @@ extern "C" int imin_estimate_decrease_noalloc(const imin_graph* g, const int32_t
     cta_slot_layout(&small);
     const uint32_t small_blocks = static_cast<uint32_t>(std::min<uint64_t>(blocks, room / small.slot_bytes));
     const uint32_t whole_blocks = static_cast<uint32_t>(std::min<uint64_t>(blocks, room / cfg.slot_bytes));
-    // Few samples per whole-graph slot are done sooner by that launch alone: the three launches'
-    // latencies add up, and a cascade that outgrows a small slot runs twice. n = 16,384 (146 slots):
-    // theta = 2,000 0.37 ms against 0.48, theta = 4,000 0.59 against 0.50; n = 50,021 (56 slots):
-    // theta = 1,000 0.52 against 0.66, theta = 2,000 1.12 against 0.67. Where the small slots hold
-    // every cascade (n = 2,000, 550 slots), theta = 2,000 0.20 against 0.21, theta = 4,000 0.28
-    // against 0.23.
-    const bool whole_only = theta <= (small.rcap < cfg.rcap ? 20u : 4u) * whole_blocks;
+    // Few samples are done sooner by the last launch alone: the launches' latencies add up, and a
+    // cascade that outgrows the warp and a small slot runs three times. Both routes were timed on six
+    // kinds of graph (Chung-Lu and R-MAT; weighted cascade, trivalency, p = 0.15) of 256 to 65,536
+    // vertices, theta = 250 to 32,000. With b whole-graph slots the times cross between 2 and 10 b for
+    // b > 375, between 1 and 13 b (mostly 500 to 2,000 samples) down to b = 146, and near 3 to 20 b
+    // below. ms with one launch / three, theta = 2,000; 8,000: n = 2,048 (b = 389), R-MAT, 216 reached
+    // 0.25 / 0.20; 0.72 / 0.37. n = 4,096 (b = 314), R-MAT trivalency, 466 reached 0.52 / 0.30;
+    // 1.78 / 0.78. n = 16,384 (b = 146), p = 0.15, 420 reached 0.82 / 0.35; 2.79 / 0.90, but R-MAT
+    // weighted cascade, 63 reached, 0.26 / 0.43; 0.65 / 0.49. n = 65,536 (b = 46), R-MAT, 207 reached
+    // 1.09 / 0.68; 3.68 / 1.47. Where most cascades outgrow the small slots the three launches lose at
+    // any theta: R-MAT trivalency at 16,384 (1,749 reached) 12 %, at 65,536 2 %; likewise where every
+    // block has a whole-graph slot and most cascades outgrow the warp (500 vertices, 177 reached) 18 %.
+    const uint32_t few = whole_blocks >= 375 ? 4 * whole_blocks : std::min(20 * whole_blocks, 2000u);
+    const bool whole_only = theta <= few;
     TierPlan warp{};
     if (!whole_only) {
         plan_tier0(g->dev, static_cast<uint32_t>(n_seeds), kDefaultCutoff, &warp);
@@ -261,6 +269,7 @@ extern "C" int imin_estimate_decrease_noalloc(const imin_graph* g, const int32_t
     k_mark_ids<<<(n_seeds + 255) / 256, 256, 0, s>>>(dseeds, n_seeds, g->n, excl, bad);
     if (n_blocked > 0) k_mark_ids<<<(n_blocked + 255) / 256, 256, 0, s>>>(dblocked, n_blocked, g->n, excl, bad);
     NA_CUDA(cudaGetLastError());
+    count_launches(n_blocked > 0 ? 2 : 1);
     uint32_t hbad = 0;
     NA_CUDA(cudaMemcpyAsync(&hbad, bad, sizeof(hbad), cudaMemcpyDeviceToHost, s));
     NA_CUDA(cudaStreamSynchronize(s));
@@ -286,11 +295,13 @@ extern "C" int imin_estimate_decrease_noalloc(const imin_graph* g, const int32_t
         NA_CUDA(launch_sample_tier(0, P, warp, nullptr, s, &warp_ran));
         small.from_list = warp_ran ? 1u : 0u;
         NA_CUDA(launch_cta_tier(P, small, small_blocks, smem, base + off_slots, s));
+        count_launches(warp_ran ? 2 : 1);
         cfg.from_list = 1;
         cfg.in_tier = kTierWhole;
     }
     cfg.out_tier = 1;  // the warp tier 1 does not run here: its list takes what nothing here holds
     NA_CUDA(launch_cta_tier(P, cfg, whole_blocks, smem, base + off_slots, s));
+    count_launches(1);
 
     RoundCtl hctl;
     NA_CUDA(cudaMemcpyAsync(&hctl, ctl, sizeof(hctl), cudaMemcpyDeviceToHost, s));

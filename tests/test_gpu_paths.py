@@ -237,3 +237,26 @@ def test_spread_in_slices(cuda_lib, monkeypatch, mib):
     want = O.spread_sets(g, [0], [], sets, theta, 4, 1)
     assert np.array_equal(cuda_lib.estimate_spread_sets(gh, [0], [], sets, theta, 4, 1), want)
     assert cuda_lib.estimate_spread(gh, [0], [5], theta, 4, 1) == int(want[0])
+
+
+@pytest.mark.parametrize("n,m,thetas", [
+    (300, 1500, [4864, 4865]),        # a whole-graph slot for each of the 1,216 resident blocks
+    (2047, 20_000, [1300, 1800]),     # 389 slots: the line is at 1,556, for slots with and without room
+    (2048, 20_000, [1300, 1800]),     # for every vertex
+    (2049, 20_000, [1300, 1800]),
+    (8192, 65_536, [2000, 2001]),     # 227 slots
+    (50_021, 400_009, [900, 1400]),   # 58 slots
+])
+def test_noalloc_route_by_samples(cuda_lib, n, m, thetas):
+    """One launch up to the rule's number of samples, three beyond it, the same counters either way."""
+    rp, col = W.chung_lu(n, m, 2.1, 71)
+    g = W.Graph(n, rp, col, W.wc_thresholds(col, n))
+    gh = cuda_lib.load_graph(g)
+    s = W.uniform_seeds(n, 12, 72)
+    launched = []
+    for theta in thetas:
+        c0 = cuda_lib.launch_count()
+        got = cuda_lib.estimate_decrease_noalloc(gh, s, [], theta, 6, 1)
+        launched.append(cuda_lib.launch_count() - c0)
+        assert np.array_equal(got, O.decrease(g, s, [], theta, 6, 1))
+    assert launched == [2, 4], launched  # the mask, then one or three tiers
