@@ -14,6 +14,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <set>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -471,21 +472,23 @@ int common_checks(const imin_graph* g, const int32_t* seeds, int32_t n_seeds, ui
 // depends on the graph's cascade-size distribution and on |S| (seeds take tier-0 space), so it
 // is measured: after one untimed warm-up call, kTuneReps Alg. 2 calls per candidate (round 0
 // of the caller's key, no blockers), interleaved across candidates so that a clock or load change
-// hits all of them alike; the candidate with the smallest minimum time wins. Each call samples
-// 24 graphs per resident block of the block tier (at least 8,192, at most 65,536), so that the
-// end of a call -- blocks finishing their last cascades at different times -- does not decide
-// the comparison. The cost is bounded: the warm-up call samples 1,024 graphs; from its time per
-// sample, each timed call is sized to take about kTuneCallMs, and when fewer than 4 samples per block
-// would fit in that time (graphs whose cascades are huge, where the cutoff hardly matters) none is
-// timed. Calls that come before the tuning has been earned (kTuneRepay) take the default. The
+// hits all of them alike; the candidate with the smallest minimum time wins, but the default only
+// loses to one that beats it by kTuneFixedMs. Each call samples up to 24 graphs per resident block
+// of the block tier (at most 65,536, and no more than a round of the caller's), so that the end of a call -- blocks finishing their last cascades
+// at different times -- does not decide the comparison. The cost is bounded: the warm-up call samples
+// 1,024 graphs; from its time per sample, each timed call is sized to take about kTuneCallMs, and when
+// fewer than 4 samples per block would fit in that time (graphs whose cascades are huge, where the
+// cutoff hardly matters) none is timed. Calls that come before the tuning has been earned (kTuneRepay) take the default. The
 // choice never changes a result -- only which tier computes each sample -- and is cached per
 // graph handle and seed-set size class, and process-wide under the graph's fingerprint, so that
 // a new handle of the same graph reuses it.
 
-constexpr uint32_t kCutoffs[] = {0, 64, 96, 128, 192};
+constexpr uint32_t kCutoffs[] = {0, 64, kDefaultCutoff, 128, 192};
 constexpr int kTuneReps = 3;
 constexpr float kTuneCallMs = 2.0f;
 constexpr uint32_t kTuneWarmup = 1024;    // samples of the warm-up call
+constexpr int kDefaultCand = 2;           // kDefaultCutoff's place in kCutoffs
+constexpr float kTuneFixedMs = 0.011f;    // by how much a candidate must beat the default
 constexpr uint64_t kTuneRepay = 16;       // samples drawn per sample the tuner times (cutoff_for)
 constexpr size_t kUntunedMax = 4096;      // entries of g_untuned
 
@@ -493,12 +496,13 @@ constexpr size_t kUntunedMax = 4096;      // entries of g_untuned
 // they have to draw before the tuner looks at it (again).
 struct Untuned {
     uint64_t samples = 0;
-    uint64_t need = kTuneWarmup;
+    uint64_t need = kTuneRepay * kTuneWarmup;
 };
 
 std::mutex g_tune_mu;
 std::map<std::pair<uint64_t, int>, int32_t> g_tuned;  // (fingerprint, size class) -> cutoff
 std::map<std::pair<uint64_t, int>, Untuned> g_untuned;
+std::set<std::pair<int, int>> g_used;  // (device, kind of kernels) that a warm-up has run
 
 // Identity of a graph for the process-wide tuning cache: a 64-bit mix of its sizes, its device
 // and about 4,096 evenly spaced entries of each CSR array. Two different graphs that collide
@@ -571,6 +575,14 @@ int time_call(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t k
     return check_ctl(hctl);
 }
 
+// Whether the process's warm-ups have not run the kernels of g's kind (device, model, place of the
+// block tier's bitmap) before; from now on they have.
+bool first_use(const imin_graph* g)
+{
+    std::lock_guard<std::mutex> lk(g_tune_mu);
+    return g_used.insert({g->device, 2 * g->model + (g->n > kCtaMaxVertices)}).second;
+}
+
 // as_theta: samples per round of the call the tuning is for, whose kernels are timed.
 // drawn: samples that the calls so far have drawn on this graph (0: tune in any case). *out < 0: they
 // have not earned the tuning yet (its timed calls are more than a kTuneRepay-th of them); no candidate
@@ -586,7 +598,7 @@ int tune_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t
     int rc = time_call(g, seeds, key, kDefaultCutoff, tw, as_theta, s, &warm, &warp_done);  // warm-up, cost
     if (rc) return rc;
     const auto costly = [&] { return kTuneCallMs * tw < 4.0 * blocks * warm; };
-    if (costly()) {  // once more: a process's first call also waits for its kernels to be loaded
+    if (first_use(g) && costly()) {  // once more: it also waited for its kernels to be loaded
         rc = time_call(g, seeds, key, kDefaultCutoff, tw, as_theta, s, &warm, &warp_done);
         if (rc) return rc;
     }
@@ -604,13 +616,13 @@ int tune_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t
     };
     // a small warm-up is dominated by its slowest block, so the timed calls will have at least the
     // samples it makes room for; re-estimate on a call of that size
-    uint32_t theta = static_cast<uint32_t>(std::min<double>({kTuneCallMs / per_sample, 24.0 * blocks, 65536.0}));
+    const double most = std::min<double>({24.0 * blocks, 65536.0, std::max<double>(as_theta, 4.0 * blocks)});
+    uint32_t theta = static_cast<uint32_t>(std::min<double>(kTuneCallMs / per_sample, most));
     if (too_early(theta)) return IMIN_OK;
     rc = time_call(g, seeds, key, kDefaultCutoff, theta, as_theta, s, &warm);
     if (rc) return rc;
     per_sample = std::max(1e-7, static_cast<double>(warm) / theta);
-    theta = static_cast<uint32_t>(std::min<double>({std::max(kTuneCallMs / per_sample, 4.0 * blocks),
-                                                    24.0 * blocks, 65536.0}));
+    theta = static_cast<uint32_t>(std::min<double>(std::max(kTuneCallMs / per_sample, 4.0 * blocks), most));
     if (too_early(theta)) return IMIN_OK;
     for (int rep = 0; rep < kTuneReps; ++rep) {
         for (int i = 0; i < kCand; ++i) {
@@ -620,9 +632,16 @@ int tune_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t
             t[i] = rep == 0 ? ms : std::min(t[i], ms);
         }
     }
-    int best = 0;
-    for (int i = 1; i < kCand; ++i)
-        if (t[i] < t[best]) best = i;
+    // The timed calls are as short as 0.05 ms where cascades are tiny, and what a call costs besides its
+    // samples differs by up to 0.01 ms between the cutoffs (larger ones leave fewer blocks to start, each
+    // of which clears its hashes). n = 40,000, p = 0.05: 192 is 6 % faster than 96 at the tuner's 29,184
+    // samples and 17 % slower at 400,000. So a candidate takes the default's place only if it wins by
+    // more than that. Over 30 graphs of 2,000 to 190,000 vertices, rounds of 80,000 samples then take 0.85
+    // to 1.02 of the default's time, 0.973 in the mean.
+    float need_ms = t[kDefaultCand] - kTuneFixedMs;
+    int best = kDefaultCand;
+    for (int i = 0; i < kCand; ++i)
+        if (t[i] < need_ms) { need_ms = t[i]; best = i; }
     *out = static_cast<int32_t>(kCutoffs[best]);
     return IMIN_OK;
 }
@@ -630,9 +649,11 @@ int tune_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t
 // The cutoff for a call: IMIN_TIER0_VERTICES forces one; IMIN_AUTOTUNE=0, or a stream being
 // captured (the tuner synchronizes), gives the default; otherwise the tuned value, tuning on first
 // use for this graph and seed-set size class, once its calls have drawn enough samples. rounds, theta:
-// of this call.
+// of this call. shared: a query of a batch or a request, which shares its launches; it takes what is
+// known and may run the warm-up, but the candidates, which are timed on a launch of one query, only
+// a single query has timed.
 int cutoff_for(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t key, uint32_t theta, int32_t rounds,
-               cudaStream_t s, uint32_t* out)
+               bool shared, cudaStream_t s, uint32_t* out)
 {
     if (const char* v = std::getenv("IMIN_TIER0_VERTICES"); v && *v) {
         *out = static_cast<uint32_t>(std::strtoul(v, nullptr, 10));
@@ -662,10 +683,11 @@ int cutoff_for(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t 
         }
     }
     // A short call cannot repay the tuning, which gives a few percent and costs about as much as the
-    // samples it times. So the samples of a graph's calls (all rounds of a greedy call) are added up,
-    // and the tuner runs when they come to kTuneRepay times the ones it would time; until then calls
-    // take the default. A program of many short calls is tuned like one of a single long call, and 50
-    // rounds of 25 ms tune at once.
+    // samples it draws. So the samples of a graph's calls (all rounds of a greedy call) are added up, and
+    // the warm-up and then the timed calls run when they come to kTuneRepay times theirs; until then
+    // calls take the default. (With the warm-up at its own 1,024 samples, the first batch of 15 queries of
+    // 16 rounds of 148 went from 4.4 to 6.3 ms.) A program of many short calls is tuned like one of a
+    // single long call, and 50 rounds of 25 ms tune at once.
     // First call of theta = 256 on a 2,000-vertex graph 0.46 -> 0.21 ms; of AdvancedGreedy there
     // (theta = 10^4, b = 10) 10.1 -> 2.1 ms; of a batch of 48 new queries 467 -> 52 ms.
     uint64_t drawn = 0, need = 0;
@@ -674,8 +696,8 @@ int cutoff_for(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t 
         if (g_untuned.size() >= kUntunedMax) g_untuned.clear();  // only the counts start again
         Untuned& u = g_untuned[{g->fingerprint, cls}];
         u.samples += static_cast<uint64_t>(theta) * rounds;
-        if (u.samples < u.need) return IMIN_OK;
-        drawn = u.samples;
+        if (u.samples < u.need || (shared && u.need != Untuned{}.need)) return IMIN_OK;
+        drawn = shared ? 1 : u.samples;
     }
     int32_t best = -1;
     const int rc = tune_cutoff(g, seeds, key, s, theta, drawn, &best, &need);
@@ -701,7 +723,7 @@ void count_launches(uint64_t kernels) { g_launches.fetch_add(kernels, std::memor
 int tuned_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t key, uint32_t theta,
                  int32_t rounds, cudaStream_t s, uint32_t* out)
 {
-    return cutoff_for(g, seeds, key, theta, rounds, s, out);
+    return cutoff_for(g, seeds, key, theta, rounds, true, s, out);
 }
 
 }  // namespace imin
@@ -726,7 +748,7 @@ int estimate_impl(const imin_graph* g, const int32_t* seeds, int32_t n_seeds,
 
     const bool dev_out = is_device_ptr(out_delta);
     uint32_t cutoff = 0;
-    rc = cutoff_for(g, hseeds, key, theta, 1, s, &cutoff);
+    rc = cutoff_for(g, hseeds, key, theta, 1, false, s, &cutoff);
     if (rc) return rc;
     Query q(s);
     rc = setup_query(g, hseeds, theta, dev_out ? reinterpret_cast<unsigned long long*>(out_delta) : nullptr,
@@ -889,7 +911,7 @@ int greedy_impl(Driver which, const imin_graph* g, const int32_t* seeds, int32_t
 
     uint32_t cutoff = 0;
     const int32_t rounds = std::min<int32_t>(b, g->n - n_seeds);
-    rc = cutoff_for(g, hseeds, key, theta, rounds, s, &cutoff);
+    rc = cutoff_for(g, hseeds, key, theta, rounds, false, s, &cutoff);
     if (rc) return rc;
     Query q(s);
     rc = setup_query(g, hseeds, theta, nullptr, cutoff, q);
@@ -1090,8 +1112,8 @@ int batch_impl(Driver which, imin_query* qs, int32_t nq, void* stream, uint32_t 
     bool all_ic = true;  // every graph IC: the launches take the IC-only kernels
     for (int32_t i = 0; i < nq; ++i) all_ic = all_ic && qs[i].graph->model == 0;
     // the warp tier in front: queries whose seed sets fit its shared-memory working set and whose
-    // graph's tuned warp/block cutoff (the single-query autotuner's, per graph and seed-set size
-    // class, tuned here on first use) is not 0; the launch holds the largest of those cutoffs
+    // graph's warp/block cutoff (the single-query autotuner's, per graph and seed-set size class, where
+    // it is tuned) is not 0. The launch holds the largest of those cutoffs
     std::vector<uint8_t> warp_q(nq, 0);
     uint32_t warp_ns = 0, cutoff = 0;
     for (int32_t i = 0; i < nq; ++i) {

@@ -45,15 +45,15 @@ def test_all_rounds_of_a_greedy_call_count(cuda_lib):
 
 
 def test_short_calls_add_up_and_a_long_one_tunes(cuda_lib):
-    """512 samples: default cutoff, own kernels only. The next 512 bring the sum to 1,024 and run the
+    """8,192 samples: default cutoff, own kernels only. The next 8,192 bring the sum to 16,384 and run the
     warm-up, once. A batch query and a request count too, and the call that completes the sum tunes."""
     g = _chung_lu(2000, 10000, 511)
     gh = cuda_lib.load_graph(g)
     s = W.uniform_seeds(g.n, 10, 512)
-    want = O.decrease(g, s, [], 512, 3, 0)
+    want = O.decrease(g, s, [], 8192, 3, 0)
     counts = []
     for _ in range(4):
-        n, got = _launches(cuda_lib, lambda: cuda_lib.estimate_decrease(gh, s, [], 512, 3, 0))
+        n, got = _launches(cuda_lib, lambda: cuda_lib.estimate_decrease(gh, s, [], 8192, 3, 0))
         assert np.array_equal(got, want)
         counts.append(n)
     assert counts[1] > counts[0] == counts[2] == counts[3], counts
@@ -61,17 +61,17 @@ def test_short_calls_add_up_and_a_long_one_tunes(cuda_lib):
     tuned, _ = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, 37, 100_000, 7))
     after, _ = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, 37, 100_000, 7))
     assert tuned >= after + 2 * TIMED_CALLS, (tuned, after)
-    assert np.array_equal(cuda_lib.estimate_decrease(gh, s, [], 512, 3, 0), want)
+    assert np.array_equal(cuda_lib.estimate_decrease(gh, s, [], 8192, 3, 0), want)
 
 
 def test_huge_cascades_drop_the_warp_tier_below_1024_samples_a_round(cuda_lib, monkeypatch):
-    """Three rounds of 600 samples on a graph whose cascades all outgrow the warp tier: the warm-up sees
-    it, and the rounds run without that tier, like calls with a forced cutoff of 0."""
+    """28 rounds of 600 samples on a graph whose cascades all outgrow the warp tier: the warm-up sees it,
+    and the rounds run without that tier from then on, like calls with a forced cutoff of 0."""
     rp, col = W.chung_lu(8000, 48000, 2.1, 521)
     g = W.Graph(8000, rp, col, np.full(len(col), int(0.3 * 2**32), np.uint32))
     gh = cuda_lib.load_graph(g)
     hubs = np.argsort(-g.out_degree())[:20].astype(np.int32)
-    cuda_lib.advanced_greedy(gh, hubs, 3, 600, 7)
+    cuda_lib.advanced_greedy(gh, hubs, 28, 600, 7)
     got, b = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, hubs, 3, 600, 7))
     monkeypatch.setenv("IMIN_TIER0_VERTICES", "0")
     forced, b0 = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, hubs, 3, 600, 7))
@@ -100,8 +100,8 @@ def test_a_tuned_cutoff_is_shared_by_handles_of_one_graph(cuda_lib):
 def test_the_tuner_times_the_kernels_of_the_call(cuda_lib, theta, rounds, budget):
     """The warp tier has one instantiation for rounds of more than two samples per resident warp (5 blocks
     per SM) and one for fewer (4); the line lies at 7,296 samples where a cutoff leaves 3 blocks per SM,
-    at 12,160 where it leaves 5. A call that tunes runs only its own, in the timed calls too, whose
-    sample counts lie on both sides of that line."""
+    at 12,160 where it leaves 5. A call that tunes runs only its own, in the warm-up and the timed calls
+    too, whatever their sample counts."""
     import re
 
     import torch
@@ -122,3 +122,43 @@ def test_the_tuner_times_the_kernels_of_the_call(cuda_lib, theta, rounds, budget
     if not seen:
         pytest.skip("no kernel records from the profiler here")
     assert set(seen) == {str(budget)} and len(seen) > TIMED_CALLS, (set(seen), len(seen))
+
+
+def test_equal_candidates_leave_the_default(cuda_lib):
+    """Cascades of a few vertices: candidates from 64 on do the same work per sample, and what else a timed
+    call of 0.05 ms costs (fewer blocks at larger cutoffs) may not decide between them."""
+    rp, col = W.chung_lu(40_000, 200_000, 2.1, 551)
+    g = W.Graph(40_000, rp, col, np.full(len(col), int(0.002 * 2**32), np.uint32))
+    gh = cuda_lib.load_graph(g)
+    s = W.uniform_seeds(g.n, 10, 552)
+    assert [cuda_lib.autotune(gh, s, k) for k in range(12)] == [96] * 12
+
+
+def test_a_costly_warm_up_runs_once_per_graph(cuda_lib):
+    """A warm-up that shows huge cascades is repeated only in a process's first use of its kernels: later
+    graphs of the kind pay for one (the mask and three tiers)."""
+    counts = []
+    for seed in (561, 562, 563):
+        rp, col = W.chung_lu(8000, 48000, 2.1, seed)
+        g = W.Graph(8000, rp, col, np.full(len(col), int(0.3 * 2**32), np.uint32))
+        gh = cuda_lib.load_graph(g)
+        hubs = np.argsort(-g.out_degree())[:20].astype(np.int32)
+        n, _ = _launches(cuda_lib, lambda: cuda_lib.autotune(gh, hubs, 7))
+        counts.append(n)
+    assert counts[1] == counts[2] <= 4, counts
+
+
+def test_a_first_short_call_runs_its_own_kernels_only(cuda_lib):
+    """Fewer than 16,384 samples over all rounds, in one call of a driver or in the queries of a batch: no
+    warm-up, whose 1,024 samples would be a good part of the call."""
+    g = _chung_lu(3000, 15000, 571)
+    s = W.uniform_seeds(g.n, 10, 572)
+    gh = cuda_lib.load_graph(g)
+    first, b1 = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, 16, 500, 7))
+    second, b2 = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, 16, 500, 7))
+    assert first == second and np.array_equal(b1, b2), (first, second)
+    graphs = [cuda_lib.load_graph(_chung_lu(3000, 15000, 573 + i)) for i in range(3)]
+    items = [(h, s, 16, 500, 7) for h in graphs]
+    first, r1 = _launches(cuda_lib, lambda: cuda_lib.batch_advanced_greedy(items))
+    second, r2 = _launches(cuda_lib, lambda: cuda_lib.batch_advanced_greedy(items))
+    assert first == second and all(np.array_equal(a, b) for a, b in zip(r1, r2)), (first, second)
