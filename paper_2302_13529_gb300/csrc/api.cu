@@ -1113,8 +1113,11 @@ int batch_impl(Driver which, imin_query* qs, int32_t nq, void* stream, uint32_t 
     for (int32_t i = 0; i < nq; ++i) all_ic = all_ic && qs[i].graph->model == 0;
     // the warp tier in front: queries whose seed sets fit its shared-memory working set and whose
     // graph's warp/block cutoff (the single-query autotuner's, per graph and seed-set size class, where
-    // it is tuned) is not 0. The launch holds the largest of those cutoffs
+    // it is tuned) is not 0. The launch has one capacity, their median by samples: a
+    // larger one leaves fewer resident blocks for all of them (256 trivalency queries, most at 96: 27.6 ms
+    // a step with 4 blocks per SM, 31.7 ms when one query's 192 left 3).
     std::vector<uint8_t> warp_q(nq, 0);
+    std::map<uint32_t, uint64_t> wanted;  // cutoff -> samples per step
     uint32_t warp_ns = 0, cutoff = 0;
     for (int32_t i = 0; i < nq; ++i) {
         if (static_cast<uint32_t>(qs[i].n_seeds) > kBatchWarpMaxSeeds) continue;
@@ -1125,8 +1128,15 @@ int batch_impl(Driver which, imin_query* qs, int32_t nq, void* stream, uint32_t 
         if (c > 0) {
             warp_q[i] = 1;
             warp_ns = std::max<uint32_t>(warp_ns, static_cast<uint32_t>(qs[i].n_seeds));
-            cutoff = std::max(cutoff, c);
+            wanted[c] += qs[i].theta;
         }
+    }
+    uint64_t all = 0, below = 0;
+    for (const auto& w : wanted) all += w.second;
+    for (const auto& w : wanted) {
+        if (2 * below >= all) break;
+        cutoff = w.first;
+        below += w.second;
     }
     TierCfg wcfg{};
     uint32_t warp_blocks = 0;

@@ -162,3 +162,25 @@ def test_a_first_short_call_runs_its_own_kernels_only(cuda_lib):
     first, r1 = _launches(cuda_lib, lambda: cuda_lib.batch_advanced_greedy(items))
     second, r2 = _launches(cuda_lib, lambda: cuda_lib.batch_advanced_greedy(items))
     assert first == second and all(np.array_equal(a, b) for a, b in zip(r1, r2)), (first, second)
+
+
+def test_one_query_of_a_batch_does_not_set_the_capacity_for_all(cuda_lib):
+    """Cascades of exactly 80 or 150 vertices besides the seeds: 96 and 192 are the smallest candidates that
+    hold them. A batch of two of the first and one of the second runs its warp launch at 96 (the
+    third query's samples go to the block tier), one of the second alone at 192."""
+    def star(leaves, n):
+        row = np.zeros(n + 1, np.int32)
+        row[1:] = leaves
+        return W.Graph(n, row, np.arange(20, 20 + leaves, dtype=np.int32), np.full(leaves, 2**32 - 1, np.uint32))
+
+    s = list(range(20))
+    graphs = [star(80, 900), star(80, 901), star(150, 902)]
+    handles = [cuda_lib.load_graph(g) for g in graphs]
+    cuts = [cuda_lib.autotune(h, s, 1) for h in handles]
+    assert cuts == [96, 96, 192], cuts
+    theta = 300
+    items = [(h, s, 1, theta, 5) for h in handles]
+    found = cuda_lib.batch_advanced_greedy(items)
+    assert list(cuda_lib.last_stats()["tier_samples"]) == [2 * theta, 0, 0, theta]
+    assert cuda_lib.batch_advanced_greedy(items[2:])[0].tolist() == found[2].tolist() == [20]
+    assert list(cuda_lib.last_stats()["tier_samples"]) == [theta, 0, 0, 0]
