@@ -46,8 +46,8 @@ struct SpreadWork {
     unsigned long long first, last;
     uint32_t grab;                      // items a warp takes at a time
     unsigned long long* sums;           // per set
-    uint32_t* handoff;                  // kHandoffWords per entry: set, sample, chunk start, queue
-                                        // length, examined and live edges (64 bits each), queue
+    uint32_t* handoff;                  // kHandoffWords per entry: set, sample, chunk start, unused,
+                                        // examined and live edges (64 bits each), the full queue
 };
 
 struct __align__(16) WarpSpread {
@@ -81,12 +81,12 @@ __device__ __forceinline__ bool insert_new(uint32_t* hash, uint32_t v)
 }
 
 // One item of the warp kernel: |R| without the seeds, or kEmpty when the queue is too small; then
-// *at is the queue index of the chunk it stopped in, *tail the queue's length, and examined and
-// live are the counts before that chunk (per lane). The hash is empty on entry and on return.
+// *at is the queue index of the chunk it stopped in, the queue is full, and examined and live are the
+// counts before that chunk (per lane). The hash is empty on entry and on return.
 template <int M>
 __device__ __forceinline__ uint32_t spread_sample(const SampleParams& P, WarpSpread& w, const int32_t* set, uint32_t k,
-                                                  uint32_t j, uint32_t lane, uint32_t* at, uint32_t* tail,
-                                                  uint32_t& examined, uint32_t& live)
+                                                  uint32_t j, uint32_t lane, uint32_t* at, uint32_t& examined,
+                                                  uint32_t& live)
 {
     // a set's vertices count as visited from the start, so nothing discovers them
     for (uint32_t i = lane; i < k; i += 32) insert_new(w.hash, static_cast<uint32_t>(set[i]));
@@ -149,7 +149,6 @@ __device__ __forceinline__ uint32_t spread_sample(const SampleParams& P, WarpSpr
         reinterpret_cast<uint4*>(w.hash)[i] = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
     __syncwarp();
     *at = head;
-    *tail = kQueue;
     return over ? kEmpty : end_q - ns;
 }
 
@@ -173,9 +172,9 @@ __global__ void __launch_bounds__(kWarps * 32, 5) k_spread_warp(SampleParams P, 
         uint32_t j = static_cast<uint32_t>((W.first + i0) % P.theta);
         unsigned long long sum = 0;
         for (uint32_t i = i0; i < i1; ++i) {
-            uint32_t ex = 0, lv = 0, at = 0, tail = 0;
+            uint32_t ex = 0, lv = 0, at = 0;
             const uint32_t found = spread_sample<M>(P, w, W.sets + static_cast<uint64_t>(set) * W.k, W.k, j, lane, &at,
-                                                    &tail, ex, lv);
+                                                    ex, lv);
             if (found != kEmpty) {
                 sum += P.ns + found;
                 reached += P.ns + found;
@@ -192,11 +191,10 @@ __global__ void __launch_bounds__(kWarps * 32, 5) k_spread_warp(SampleParams P, 
                     h[0] = set;
                     h[1] = j;
                     h[2] = at;
-                    h[3] = tail;
                     *reinterpret_cast<unsigned long long*>(h + 4) = exs;
                     *reinterpret_cast<unsigned long long*>(h + 6) = lvs;
                 }
-                for (uint32_t t = lane; t < tail; t += 32) h[kHeader + t] = w.queue[t];
+                for (uint32_t t = lane; t < kQueue; t += 32) h[kHeader + t] = w.queue[t];
                 __syncwarp();
             }
             if (++j == P.theta || i + 1 == i1) {
@@ -252,7 +250,7 @@ k_spread_block(SampleParams P, CtaCfg C, SpreadWork W)
         __syncthreads();
         if (sh.item >= count) break;
         const uint32_t* h = W.handoff + static_cast<uint64_t>(sh.item) * kHandoffWords;
-        const uint32_t set = h[0], at = h[2], found = P.ns + h[3];
+        const uint32_t set = h[0], at = h[2], found = P.ns + kQueue;
         // a slot of a large graph holds at most 2^18 ids, and the warp left the vertices it could not
         // queue for the block to find: a cascade that does not fit already will not fit later
         if (1 + found > C.rcap) {

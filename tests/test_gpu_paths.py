@@ -260,3 +260,18 @@ def test_noalloc_route_by_samples(cuda_lib, n, m, thetas):
         launched.append(cuda_lib.launch_count() - c0)
         assert np.array_equal(got, O.decrease(g, s, [], theta, 6, 1))
     assert launched == [2, 4], launched  # the mask, then one or three tiers
+
+
+@pytest.mark.parametrize("model", ["ic", "lt"])
+@pytest.mark.parametrize("cutoff", ["64", "192"])
+def test_few_and_many_samples_per_warp(cuda_lib, monkeypatch, model, cutoff):
+    """Both register budgets of the warp tier on one graph: the line is at two samples per resident warp,
+    12,160 with 5 blocks per SM and 7,296 with 3."""
+    rp, col = W.chung_lu(1500, 7000, 2.1, 81)
+    g = W.Graph(1500, rp, col, W.lt_wc_weights(col, 1500) if model == "lt" else W.wc_thresholds(col, 1500))
+    monkeypatch.setenv("IMIN_TIER0_VERTICES", cutoff)
+    gh = cuda_lib.load_graph(g, model=model)
+    s = W.uniform_seeds(g.n, 100, 82)
+    for theta in (7296, 7297, 9728, 9729, 12160, 12161):
+        want = O.decrease(g, s, [], theta, 6, 1, model=model)
+        assert np.array_equal(cuda_lib.estimate_decrease(gh, s, [], theta, 6, 1), want)
