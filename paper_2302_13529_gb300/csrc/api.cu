@@ -324,7 +324,8 @@ int setup_query(const imin_graph* g, const std::vector<int32_t>& seeds, uint32_t
     // with the warp tier in front of the block tier, one hand-off snapshot per sample it may give
     // up on, after the block tier's slots: the block tier resumes those samples where it stopped
     uint64_t handoff_bytes = 0;
-    if (q.plan.use_cta && q.plan.cta.from_list && q.plan.blocks[0] > 0) {
+    if (q.plan.use_cta && q.plan.cta.from_list && q.plan.blocks[0] > 0 &&
+        slot_holds_handoffs(q.plan.cta, q.plan.cfg[0], static_cast<uint32_t>(g->n), static_cast<uint32_t>(g->m))) {
         const Handoff h = handoff_layout(q.plan.cfg[0].rcap, q.plan.cfg[0].dcap, q.plan.cfg[0].ecap);
         q.plan.cta.handoff_stride = h.stride;
         handoff_bytes = static_cast<uint64_t>(theta) * h.stride;
@@ -1192,7 +1193,11 @@ int batch_impl(Driver which, imin_query* qs, int32_t nq, void* stream, uint32_t 
     uint64_t warp_theta = 0;
     for (int32_t i = 0; i < nq; ++i)
         if (warp_q[i]) warp_theta += qs[i].theta;
-    if (warp_theta > 0) {
+    bool held = warp_theta > 0;
+    for (int k = 0; k < kBatchClasses; ++k)
+        held = held && (cls_n[k] == 0 || slot_holds_handoffs(cfg[k], wcfg, static_cast<uint32_t>(cls_n[k]),
+                                                             static_cast<uint32_t>(cls_m[k])));
+    if (held) {
         const Handoff h = handoff_layout(wcfg.rcap, wcfg.dcap, wcfg.ecap);
         handoff_stride = h.stride;
         handoff_cap = static_cast<uint32_t>(

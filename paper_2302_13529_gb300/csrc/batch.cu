@@ -79,6 +79,20 @@ __device__ __forceinline__ SampleParams params_of(const BatchQuery& Q, uint32_t 
     return P;
 }
 
+// One thread: the samples of a work item whose seeds no slot holds go to the whole-graph tier.
+__device__ __forceinline__ void pass_on_item(const BatchStep& B, uint32_t q, unsigned long long item)
+{
+    const BatchQuery& Q = B.q[q];
+    const unsigned long long j0 = (item - B.prefix[q]) * B.chunk;
+    const unsigned long long j1 = min(j0 + B.chunk, static_cast<unsigned long long>(Q.theta));
+    for (unsigned long long j = j0; j < j1; ++j) {
+        if (Q.done != nullptr && Q.done[j] != 0) continue;
+        const uint32_t p = atomicAdd(&B.ctl->over_count, 1u);
+        if (p < B.over_cap) B.over[p] = make_uint2(q, static_cast<uint32_t>(j));
+        else atomicOr(&B.ctl->error, kErrCapacity);
+    }
+}
+
 template <bool kSmemBitmap, int M>
 __global__ void __launch_bounds__(cta_threads<kSmemBitmap>(), 1024 / cta_threads<kSmemBitmap>()) k_batch_cta(BatchStep B, CtaCfg C)
 {
@@ -115,6 +129,10 @@ __global__ void __launch_bounds__(cta_threads<kSmemBitmap>(), 1024 / cta_threads
                 bool ph2;
                 s_q = q;
                 s_skip = !step_active(B.q[q], B, &pos, &ph2);
+                if (!s_skip && !seeds_fit(B.q[q].ns, C)) {
+                    pass_on_item(B, q, item);
+                    s_skip = 1;
+                }
             }
         }
         __syncthreads();
@@ -158,10 +176,9 @@ __global__ void __launch_bounds__(cta_threads<kSmemBitmap>(), 1024 / cta_threads
             const uint32_t j = hdr[0], q = hdr[8];
             const SampleParams P = params_of(B.q[q], B.step - B.q[q].start);
             uint32_t from[3];
-            int rc = kSampleOverflow;
-            if (restore_handoff<kCtaThreads>(P, C, hb, S, bm, sh, tid, from))
-                rc = run_sample_cta<kSmemBitmap, false, M>(P, C, bm, dsm, sh, S, j, tid, sc, examined, live,
-                                                           ExtraBlocked{nullptr, 0u}, from);
+            restore_handoff<kCtaThreads>(P, hb, S, bm, sh, tid, from);
+            const int rc = run_sample_cta<kSmemBitmap, false, M>(P, C, bm, dsm, sh, S, j, tid, sc, examined, live,
+                                                                 ExtraBlocked{nullptr, 0u}, from);
             if (tid == 0) {
                 if (rc == kSampleOverflow) {
                     const uint32_t p = atomicAdd(&B.ctl->over_count, 1u);

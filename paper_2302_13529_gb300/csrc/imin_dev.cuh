@@ -8,15 +8,16 @@
 //      into groups of 4 consecutive edge ids; each lane takes one group, loads its 4
 //      thresholds with one 16-byte load and evaluates one Philox4x32-10 call whose 4 output words
 //      decide the 4 edges. The ids of live edges wait in shared memory until 32 of them (or the
-//      chunk's last) can be visited with a lane each: the target is loaded only then. This kernel
-//      is bound by instruction issue, and with a few percent of the edges live, visiting them as
-//      they came left most lanes idle: 48 queries of the trivalency batch 36.3 -> 29.0 ms in the
-//      warp tier, the mid workload 33.2 -> 32.5 ms. Targets that are
-//      neither seeds nor blocked go through a warp-shared open-addressing hash (global id ->
-//      local id). A newly inserted vertex gets the next local id, so local ids follow BFS
-//      discovery order and every level occupies a contiguous id range; the discovering vertex
-//      becomes its initial dominator candidate. Live edges to already-known vertices are kept
-//      as "non-tree" edges.
+//      chunk's last) can be visited with a lane each: the target is loaded only then. With a few
+//      percent of the edges live, visiting them as they came left most lanes idle: 48 queries of
+//      the trivalency batch 36.3 -> 29.0 ms in the warp tier, the mid workload 33.2 -> 32.5 ms.
+//      What bounds the kernel: on the mid workload instruction issue (79 % of the slots); in the
+//      batch issue together with the residency that shared memory leaves (71 % of the slots with
+//      4 blocks per SM at cutoff 96, 60 % with 3 at cutoff 192). Targets that are neither seeds
+//      nor blocked go through a warp-shared open-addressing hash (global id -> local id). A newly
+//      inserted vertex gets the next local id, so local ids follow BFS discovery order and every
+//      level occupies a contiguous id range; the discovering vertex becomes its initial dominator
+//      candidate. Live edges to already-known vertices are kept as "non-tree" edges.
 //   2. immediate dominators (Defs. 5-6) by the iterative intersection scheme of Cooper,
 //      Harvey and Kennedy on BFS numbering: start from the BFS tree and, for every non-tree
 //      edge (p, v), lower idom(v) to the nearest common ancestor of idom(v), p and v's BFS
@@ -222,6 +223,19 @@ struct CtaCfg {
     uint32_t out_tier;    // tier whose list receives the samples that do not fit (kTierWhole)
 };
 
+// Whether a block's slot holds the seeds (and id 0): always, unless more than 2^18 - 2 of them meet the
+// vertex cap of a large graph's slots.
+__host__ __device__ inline bool seeds_fit(uint32_t ns, const CtaCfg& c) { return 1 + ns <= c.rcap; }
+
+// Whether a block's slot holds every hand-off that a warp tier of these capacities leaves on a graph of
+// n vertices and m edges: always, unless the slot's capacities are lowered below the warp tier's own.
+// Without hand-offs the block tier runs the samples from the start. (With this and seeds_fit tested in
+// the block kernel for each sample, it took 1.2-1.5 % longer under trivalency and linear threshold.)
+__host__ __device__ inline bool slot_holds_handoffs(const CtaCfg& c, const TierCfg& warp, uint32_t n, uint32_t m)
+{
+    return c.rcap >= (warp.rcap < n + 1 ? warp.rcap : n + 1) && c.ecap >= (warp.ecap < m ? warp.ecap : m);
+}
+
 // One query of a batch (batch.cu): its graph, seed set, masks, counters and results.
 struct BatchQuery {
     DevGraph g;
@@ -312,9 +326,9 @@ __host__ __device__ inline WarpLayout warp_layout(uint32_t rcap, uint32_t hcap, 
     return L;
 }
 
-// Shared-memory work area of one warp's frontier chunk (always shared memory).
-// The non-empty rows of up to 32 frontier vertices, in order, and the live edges that wait to be
-// visited: at most 31 left over plus one iteration's 32 lanes x 4 edges.
+// One warp's work area for a frontier chunk, in shared memory in every tier: the non-empty rows of up
+// to 32 frontier vertices, in order, and the live edges that wait to be visited, at most 31 left over
+// plus one iteration's 32 lanes x 4 edges.
 constexpr uint32_t kStageCap = 160;
 struct __align__(16) WarpStage {
     uint32_t edge[kStageCap];  // live edge ids

@@ -149,8 +149,9 @@ cudaError_t launch_batch_warp(const BatchStep& B, const TierCfg& c, uint32_t blo
                               cudaStream_t s);
 // The warp/block cutoff of one query (api.cu): IMIN_TIER0_VERTICES when set; kDefaultCutoff with
 // IMIN_AUTOTUNE=0 or on a capturing stream; otherwise the autotuner's value for the graph and the
-// seed-set size class, tuned on `s` and cached once the calls on them, this one of `rounds` rounds of
-// theta samples included, have drawn enough to repay it (kDefaultCutoff until then).
+// seed-set size class where a single query or imin_autotune has tuned them, or 0 where the warm-up, run
+// on `s` once the calls on them (this one of `rounds` rounds of theta samples included) have drawn
+// enough, shows huge cascades; else kDefaultCutoff.
 int tuned_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t key, uint32_t theta,
                  int32_t rounds, cudaStream_t s, uint32_t* out);
 

@@ -56,10 +56,9 @@ __global__ void __launch_bounds__(cta_threads<kSmemBitmap>(), 1024 / cta_threads
             const uint8_t* hb = C.scratch + static_cast<uint64_t>(gridDim.x) * C.slot_bytes +
                                 static_cast<uint64_t>(sh.item) * C.handoff_stride;
             uint32_t from[3];
-            rc = kSampleOverflow;
-            if (restore_handoff<kCtaThreads>(P, C, hb, S, bm, sh, tid, from))
-                rc = run_sample_cta<kSmemBitmap, false, M>(P, C, bm, dsm, sh, S, j, tid, sc, examined, live,
-                                                           ExtraBlocked{nullptr, 0u}, from);
+            restore_handoff<kCtaThreads>(P, hb, S, bm, sh, tid, from);
+            rc = run_sample_cta<kSmemBitmap, false, M>(P, C, bm, dsm, sh, S, j, tid, sc, examined, live,
+                                                       ExtraBlocked{nullptr, 0u}, from);
         } else {
             rc = run_sample_cta<kSmemBitmap, false, M>(P, C, bm, dsm, sh, S, j, tid, sc, examined, live);
         }
@@ -94,6 +93,16 @@ __global__ void __launch_bounds__(cta_threads<kSmemBitmap>(), 1024 / cta_threads
             atomicAdd(st + kStPasses, sc.passes);
         }
     }
+}
+
+// In place of k_sample_cta where no sample fits a slot: all of them go to the next tier.
+__global__ void __launch_bounds__(256) k_pass_on(SampleParams P, CtaCfg C)
+{
+    if (P.done != nullptr && *P.done != 0) return;
+    const uint32_t total = C.from_list ? P.ctl->count[C.in_tier] : P.theta;
+    for (uint64_t i = blockIdx.x * 256u + threadIdx.x; i < total; i += gridDim.x * 256u)
+        P.lists[C.out_tier * P.theta + i] = C.from_list ? P.lists[C.in_tier * P.theta + i] : static_cast<uint32_t>(i);
+    if (blockIdx.x == 0 && threadIdx.x == 0) P.ctl->count[C.out_tier] = total;
 }
 
 }  // namespace
@@ -176,7 +185,9 @@ cudaError_t launch_cta_tier(const SampleParams& P, const CtaCfg& c, uint32_t blo
     CtaCfg cfg = c;
     cfg.scratch = scratch;
     const bool lt = P.g.lo4 != nullptr;
-    if (c.global_bitmap) {
+    if (!seeds_fit(P.ns, c)) {
+        k_pass_on<<<blocks, 256, 0, s>>>(P, cfg);
+    } else if (c.global_bitmap) {
         if (lt) k_sample_cta<false, kModelLT><<<blocks, cta_threads<false>(), smem, s>>>(P, cfg);
         else k_sample_cta<false, kModelIC><<<blocks, cta_threads<false>(), smem, s>>>(P, cfg);
     } else {

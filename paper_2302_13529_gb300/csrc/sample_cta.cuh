@@ -401,17 +401,14 @@ __device__ __forceinline__ void tree_sweep_packed(const SampleParams& P, CtaShar
 // bitmap and into sh, and sets from = (lb, le, nlev) for run_sample_cta: the sample continues
 // at the start of the level the warp tier could not hold, with the ids, parents, level offsets
 // and non-tree edges the warp tier had found before it. Ids are in the warp tier's discovery
-// order, which is a BFS order like the block tier's own. Returns false, with nothing written, when
-// the snapshot does not fit the slot (capacities lowered below the warp tier's own): the sample is
-// then one that the block tier cannot hold.
+// order, which is a BFS order like the block tier's own. The snapshot fits the slot: the host asks the
+// warp tier for hand-offs only where every one does (slot_holds_handoffs).
 template <uint32_t T>
-__device__ __forceinline__ bool restore_handoff(const SampleParams& P, const CtaCfg& C, const uint8_t* hb,
-                                                const Slot& S, uint32_t* bm, CtaShared<T>& sh, uint32_t tid,
-                                                uint32_t from[3])
+__device__ __forceinline__ void restore_handoff(const SampleParams& P, const uint8_t* hb, const Slot& S,
+                                                uint32_t* bm, CtaShared<T>& sh, uint32_t tid, uint32_t from[3])
 {
     const uint32_t* hdr = reinterpret_cast<const uint32_t*>(hb);
     const uint32_t lb = hdr[1], le = hdr[2], nlev = min(hdr[3], kCtaLevels), ne = hdr[4];
-    if (le > C.rcap || ne > C.ecap) return false;
     const int32_t* hg = reinterpret_cast<const int32_t*>(hb + hdr[5]);
     const uint32_t* hp = reinterpret_cast<const uint32_t*>(hb + hdr[6]);
     const uint2* he = reinterpret_cast<const uint2*>(hb + hdr[7]);
@@ -441,7 +438,6 @@ __device__ __forceinline__ bool restore_handoff(const SampleParams& P, const Cta
     from[1] = le;
     from[2] = nlev;
     __syncthreads();
-    return true;
 }
 
 // bm: visited bitmap (shared or global memory); res: 2 * C.res_slots words of shared memory for
@@ -449,7 +445,7 @@ __device__ __forceinline__ bool restore_handoff(const SampleParams& P, const Cta
 // kSpread: only the BFS; |R| (seeds included) is added to sc.reached and the dominator step is
 // skipped (the Monte-Carlo spread estimate of Def. 3); xb lists vertices blocked in this sample
 // only (reachability mode). `from` (lb, le, nlev) resumes a sample at the start of a level whose
-// state the caller restored (restore_handoff).
+// state the caller restored (restore_handoff); without it the slot must hold the seeds (seeds_fit).
 template <bool kResInBitmap, bool kSpread = false, int M = kModelAny, uint32_t T>
 __device__ __forceinline__ int run_sample_cta(const SampleParams& P, const CtaCfg& C, uint32_t* bm,
                                               uint32_t* res, CtaShared<T>& sh, const Slot& S, uint32_t j,
@@ -465,7 +461,6 @@ __device__ __forceinline__ int run_sample_cta(const SampleParams& P, const CtaCf
     const uint32_t lane = tid & 31, wid = __shfl_sync(kFull, tid >> 5, 0);
     uint32_t lb = 1, le = 1 + ns, nlev = 1;
     if (from == nullptr) {
-        if (le > C.rcap) return kSampleOverflow;  // the seeds alone outgrow a large graph's slot
         for (uint32_t i = tid; i < ns; i += kCtaThreads) {
             const int32_t u = P.seeds[i];
             S.gid[1 + i] = u;
