@@ -46,8 +46,8 @@ struct SpreadWork {
     unsigned long long first, last;
     uint32_t grab;                      // items a warp takes at a time
     unsigned long long* sums;           // per set
-    uint32_t* handoff;                  // kHandoffWords per entry: set, sample, chunk start, unused,
-                                        // examined and live edges (64 bits each), the full queue
+    uint32_t* handoff;                  // kHandoffWords per entry: set, sample, chunk start, queue
+                                        // length (kQueue), examined and live edges (64 bits each), queue
 };
 
 struct __align__(16) WarpSpread {
@@ -191,6 +191,7 @@ __global__ void __launch_bounds__(kWarps * 32, 5) k_spread_warp(SampleParams P, 
                     h[0] = set;
                     h[1] = j;
                     h[2] = at;
+                    h[3] = kQueue;
                     *reinterpret_cast<unsigned long long*>(h + 4) = exs;
                     *reinterpret_cast<unsigned long long*>(h + 6) = lvs;
                 }
@@ -250,13 +251,7 @@ k_spread_block(SampleParams P, CtaCfg C, SpreadWork W)
         __syncthreads();
         if (sh.item >= count) break;
         const uint32_t* h = W.handoff + static_cast<uint64_t>(sh.item) * kHandoffWords;
-        const uint32_t set = h[0], at = h[2], found = P.ns + kQueue;
-        // a slot of a large graph holds at most 2^18 ids, and the warp left the vertices it could not
-        // queue for the block to find: a cascade that does not fit already will not fit later
-        if (1 + found > C.rcap) {
-            if (tid == 0) atomicOr(&P.ctl->error, kErrCapacity);
-            continue;
-        }
+        const uint32_t set = h[0], at = h[2], found = P.ns + h[3];
         // slot ids start at 1, as in Alg. 2's slots
         for (uint32_t i = tid; i < found; i += kCtaThreads) {
             const uint32_t v = i < P.ns ? static_cast<uint32_t>(P.seeds[i]) : h[kHeader + i - P.ns];
@@ -305,12 +300,20 @@ k_spread_block(SampleParams P, CtaCfg C, SpreadWork W)
     }
 }
 
+// In place of k_spread_block where no hand-off fits a slot: a slot of a large graph holds at most 2^18
+// ids, and a cascade that has outgrown it will not fit later.
+__global__ void k_spread_refuse(RoundCtl* ctl)
+{
+    if (ctl->count[kTierCta] > 0) atomicOr(&ctl->error, kErrCapacity);
+}
+
 template <int M>
 cudaError_t launch_slice(const SampleParams& P, const CtaCfg& cfg, uint32_t warp_blocks, uint32_t blocks,
                          uint64_t smem, const SpreadWork& W, cudaStream_t s)
 {
     k_spread_warp<M><<<warp_blocks, kWarps * 32, 0, s>>>(P, W);
-    if (cfg.global_bitmap) k_spread_block<false, M><<<blocks, cta_threads<false>(), smem, s>>>(P, cfg, W);
+    if (1 + P.ns + kQueue > cfg.rcap && cfg.rcap <= static_cast<uint32_t>(P.g.n)) k_spread_refuse<<<1, 1, 0, s>>>(P.ctl);
+    else if (cfg.global_bitmap) k_spread_block<false, M><<<blocks, cta_threads<false>(), smem, s>>>(P, cfg, W);
     else k_spread_block<true, M><<<blocks, cta_threads<true>(), smem, s>>>(P, cfg, W);
     return cudaGetLastError();
 }
