@@ -350,22 +350,23 @@ int imin_estimate_decrease_stats(const imin_graph* g, const int32_t* seeds, int3
  * finished by the warp-per-sample tier; larger ones are re-run by the block-per-sample tier.
  * After untimed warm-up calls that estimate the time per sample, the tuner times three Alg. 2
  * calls (round 0 of `key`, no blockers; each sized to take about 2 ms, at most 24 samples per
- * resident block of the block tier and at most 65,536; in the lazy tuning at most the caller's
- * theta, but 4 per block) for each candidate cutoff
+ * resident block of the block tier and at most 65,536) for each candidate cutoff
  * {0, 64, 96, 128, 192} (0 = block tier only), interleaved, and keeps the candidate with the
- * smallest minimum time, or 96 where none is faster than it by 11 us. When fewer than 4 samples per block fit in 2 ms (huge cascades), it does
- * not time the candidates: it keeps 96 if the warm-up's warp tier finished at least a tenth of
- * its samples, and 0 otherwise. The first warm-up call samples 1,024 graphs.
+ * smallest minimum time, or 96 where none is faster than it by 20 us. When fewer than 4 samples
+ * per block fit in 2 ms (huge cascades), it does not time the candidates: it keeps 96 if the
+ * warm-up's warp tier finished at least a tenth of its samples, and 0 otherwise. The first warm-up
+ * call samples 1,024 graphs.
  * The cutoff never changes any result of this library, only which kernel computes a sample.
  * The estimate and greedy calls tune lazily for each graph and seed-set size class
  * (ceil(log2 n_seeds)) unless IMIN_AUTOTUNE=0 (fixed cutoff 96) or IMIN_TIER0_VERTICES=<c>
  * (forced cutoff c); a call on a stream under capture uses 96. The samples of the calls on a graph
- * and class (b * theta of a greedy call) are added up: the first warm-up runs at 16,384, and
- * the candidates are timed when the sum comes to 16 times the samples of the timed calls (at most
- * 16 * 15 * 65,536). Until then calls use 96. Batched queries and requests count and run the warm-up,
- * but only a single-query call times the candidates. Results and sums are kept for the
- * life of the process under a fingerprint of the graph (its sizes and sampled CSR entries), so a
- * new handle of the same graph does not tune again. This entry point re-tunes unconditionally.
+ * and class (b * theta of a greedy call) are added up: the first warm-up runs at 16,384, or with
+ * the first round of 1,024 or more, and the candidates are timed, in calls of the caller's theta (from
+ * 4 samples per block to 65,536), when the sum comes to 16 times the samples of the timed calls.
+ * Until then calls use 96. Batched queries and requests count and run the warm-up, but only a
+ * single-query call times the candidates. Results and sums are kept for the life of the process
+ * under a fingerprint of the graph (its sizes and sampled CSR entries), so a new handle of the same
+ * graph does not tune again. This entry point re-tunes unconditionally.
  *   seeds     int32[n_seeds], host or device, distinct ids in [0, n).
  *   key       Philox key of the timed calls.
  *   stream    CUDA stream (NULL: legacy default); synchronized.

@@ -474,12 +474,12 @@ int common_checks(const imin_graph* g, const int32_t* seeds, int32_t n_seeds, ui
 // is measured: after one untimed warm-up call, kTuneReps Alg. 2 calls per candidate (round 0
 // of the caller's key, no blockers), interleaved across candidates so that a clock or load change
 // hits all of them alike; the candidate with the smallest minimum time wins, but the default only
-// loses to one that beats it by kTuneFixedMs. Each call samples up to 24 graphs per resident block
-// of the block tier (at most 65,536, and no more than a round of the caller's), so that the end of a call -- blocks finishing their last cascades
-// at different times -- does not decide the comparison. The cost is bounded: the warm-up call samples
-// 1,024 graphs; from its time per sample, each timed call is sized to take about kTuneCallMs, and when
-// fewer than 4 samples per block would fit in that time (graphs whose cascades are huge, where the
-// cutoff hardly matters) none is timed. Calls that come before the tuning has been earned (kTuneRepay) take the default. The
+// loses to one that beats it by kTuneFixedMs. A call that tunes times rounds of its own size (4 samples
+// per resident block of the block tier to 65,536), imin_autotune rounds of about kTuneCallMs (at most 24
+// per block), so that the end of a round -- blocks finishing their last cascades at different times -- does
+// not decide the comparison. The cost is bounded: the warm-up call samples 1,024 graphs, and when fewer
+// than 4 samples per block would fit in kTuneCallMs by its time per sample (graphs whose cascades are
+// huge, where the cutoff hardly matters) none is timed. Calls that come before the tuning has been earned (kTuneRepay) take the default. The
 // choice never changes a result -- only which tier computes each sample -- and is cached per
 // graph handle and seed-set size class, and process-wide under the graph's fingerprint, so that
 // a new handle of the same graph reuses it.
@@ -489,7 +489,7 @@ constexpr int kTuneReps = 3;
 constexpr float kTuneCallMs = 2.0f;
 constexpr uint32_t kTuneWarmup = 1024;    // samples of the warm-up call
 constexpr int kDefaultCand = 2;           // kDefaultCutoff's place in kCutoffs
-constexpr float kTuneFixedMs = 0.011f;    // by how much a candidate must beat the default
+constexpr float kTuneFixedMs = 0.02f;     // by how much a candidate must beat the default
 constexpr uint64_t kTuneRepay = 16;       // samples drawn per sample the tuner times (cutoff_for)
 constexpr size_t kUntunedMax = 4096;      // entries of g_untuned
 
@@ -615,16 +615,22 @@ int tune_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t
         *need = kTuneRepay * kTuneReps * kCand * timed;
         return drawn > 0 && drawn < *need;
     };
-    // a small warm-up is dominated by its slowest block, so the timed calls will have at least the
-    // samples it makes room for; re-estimate on a call of that size
-    const double most = std::min<double>({24.0 * blocks, 65536.0, std::max<double>(as_theta, 4.0 * blocks)});
-    uint32_t theta = static_cast<uint32_t>(std::min<double>(kTuneCallMs / per_sample, most));
-    if (too_early(theta)) return IMIN_OK;
-    rc = time_call(g, seeds, key, kDefaultCutoff, theta, as_theta, s, &warm);
-    if (rc) return rc;
-    per_sample = std::max(1e-7, static_cast<double>(warm) / theta);
-    theta = static_cast<uint32_t>(std::min<double>(std::max(kTuneCallMs / per_sample, 4.0 * blocks), most));
-    if (too_early(theta)) return IMIN_OK;
+    uint32_t theta = 0;
+    if (as_theta != UINT32_MAX) {
+        // a round of the caller's: in a shorter one its end counts for more. R-MAT 2^18, |S| = 11: a cutoff
+        // of 0 won by 2 % at 13,000 samples, and took 4 % longer in rounds of 57,000
+        theta = std::max(std::min(as_theta, 65536u), 4 * blocks);
+        if (too_early(theta)) return IMIN_OK;
+    } else {
+        // a small warm-up is dominated by its slowest block, so the timed calls will have at least the
+        // samples it makes room for; re-estimate on a call of that size
+        const double most = std::min(24.0 * blocks, 65536.0);
+        theta = static_cast<uint32_t>(std::min(kTuneCallMs / per_sample, most));
+        rc = time_call(g, seeds, key, kDefaultCutoff, theta, as_theta, s, &warm);
+        if (rc) return rc;
+        per_sample = std::max(1e-7, static_cast<double>(warm) / theta);
+        theta = static_cast<uint32_t>(std::min(std::max(kTuneCallMs / per_sample, 4.0 * blocks), most));
+    }
     for (int rep = 0; rep < kTuneReps; ++rep) {
         for (int i = 0; i < kCand; ++i) {
             float ms = 0.f;
@@ -635,10 +641,12 @@ int tune_cutoff(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t
     }
     // The timed calls are as short as 0.05 ms where cascades are tiny, and what a call costs besides its
     // samples differs by up to 0.01 ms between the cutoffs (larger ones leave fewer blocks to start, each
-    // of which clears its hashes). n = 40,000, p = 0.05: 192 is 6 % faster than 96 at the tuner's 29,184
-    // samples and 17 % slower at 400,000. So a candidate takes the default's place only if it wins by
-    // more than that. Over 30 graphs of 2,000 to 190,000 vertices, rounds of 80,000 samples then take 0.85
-    // to 1.02 of the default's time, 0.973 in the mean.
+    // of which clears its hashes). n = 40,000, p = 0.05: 192 is 6 % faster than 96 at 29,184 samples and
+    // 17 % slower at 400,000. The cascades of later rounds are smaller, too: n = 2,000, rounds of 10^4: 192
+    // won by 11 us of 310, and the ten rounds of a greedy call take 12 % longer with it. So a candidate
+    // takes the default's place only if it wins by more than that. Over 30 graphs of 2,000 to 190,000
+    // vertices, timed at 29,184 samples, rounds of 80,000 then take 0.85 to 1.00 of the default's time,
+    // 0.974 in the mean.
     float need_ms = t[kDefaultCand] - kTuneFixedMs;
     int best = kDefaultCand;
     for (int i = 0; i < kCand; ++i)
@@ -685,9 +693,10 @@ int cutoff_for(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t 
     }
     // A short call cannot repay the tuning, which gives a few percent and costs about as much as the
     // samples it draws. So the samples of a graph's calls (all rounds of a greedy call) are added up, and
-    // the warm-up and then the timed calls run when they come to kTuneRepay times theirs; until then
-    // calls take the default. (With the warm-up at its own 1,024 samples, the first batch of 15 queries of
-    // 16 rounds of 148 went from 4.4 to 6.3 ms.) A program of many short calls is tuned like one of a
+    // the timed calls run when they come to kTuneRepay times theirs; until then calls take the default. The
+    // warm-up runs with the first round that is no shorter than it, or when shorter ones come to
+    // kTuneRepay times its samples. (With 1,024 of those, the first batch of 15 queries of 16 rounds of
+    // 148 went from 4.4 to 6.3 ms.) A program of many short calls is tuned like one of a
     // single long call, and 50 rounds of 25 ms tune at once.
     // First call of theta = 256 on a 2,000-vertex graph 0.46 -> 0.21 ms; of AdvancedGreedy there
     // (theta = 10^4, b = 10) 10.1 -> 2.1 ms; of a batch of 48 new queries 467 -> 52 ms.
@@ -697,7 +706,8 @@ int cutoff_for(const imin_graph* g, const std::vector<int32_t>& seeds, uint64_t 
         if (g_untuned.size() >= kUntunedMax) g_untuned.clear();  // only the counts start again
         Untuned& u = g_untuned[{g->fingerprint, cls}];
         u.samples += static_cast<uint64_t>(theta) * rounds;
-        if (u.samples < u.need || (shared && u.need != Untuned{}.need)) return IMIN_OK;
+        const bool warmed = u.need != Untuned{}.need;
+        if (warmed ? shared || u.samples < u.need : theta < kTuneWarmup && u.samples < u.need) return IMIN_OK;
         drawn = shared ? 1 : u.samples;
     }
     int32_t best = -1;

@@ -32,36 +32,36 @@ def _chung_lu(n, m, seed):
 
 
 def test_all_rounds_of_a_greedy_call_count(cuda_lib):
-    """71 rounds of 10^5 samples, each far shorter than the tuning, are more than 16 times the samples
-    it times (15 calls of at most 24 per resident block): the first call tunes."""
+    """160 rounds of 10^5 samples, each far shorter than the tuning, are more than 16 times the samples it
+    times (15 calls of 65,536): the first call tunes."""
     g = _chung_lu(2000, 10000, 501)
     gh = cuda_lib.load_graph(g)
     s = W.uniform_seeds(g.n, 10, 502)
-    first, b1 = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, 71, 100_000, 7))
-    second, b2 = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, 71, 100_000, 7))
-    third, b3 = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, 71, 100_000, 7))
+    first, b1 = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, 160, 100_000, 7))
+    second, b2 = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, 160, 100_000, 7))
+    third, b3 = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, 160, 100_000, 7))
     assert first >= second + 2 * TIMED_CALLS and second == third, (first, second, third)
     assert np.array_equal(b1, b2) and np.array_equal(b2, b3)
 
 
 def test_short_calls_add_up_and_a_long_one_tunes(cuda_lib):
-    """8,192 samples: default cutoff, own kernels only. The next 8,192 bring the sum to 16,384 and run the
-    warm-up, once. A batch query and a request count too, and the call that completes the sum tunes."""
+    """Calls of 1,000 samples: default cutoff, own kernels only. The 17th brings the sum past 16,384 and runs
+    the warm-up, once. A batch query and a request count too, and the call that completes the sum tunes."""
     g = _chung_lu(2000, 10000, 511)
     gh = cuda_lib.load_graph(g)
     s = W.uniform_seeds(g.n, 10, 512)
-    want = O.decrease(g, s, [], 8192, 3, 0)
+    want = O.decrease(g, s, [], 1000, 3, 0)
     counts = []
-    for _ in range(4):
-        n, got = _launches(cuda_lib, lambda: cuda_lib.estimate_decrease(gh, s, [], 8192, 3, 0))
+    for _ in range(20):
+        n, got = _launches(cuda_lib, lambda: cuda_lib.estimate_decrease(gh, s, [], 1000, 3, 0))
         assert np.array_equal(got, want)
         counts.append(n)
-    assert counts[1] > counts[0] == counts[2] == counts[3], counts
-    cuda_lib.batch_advanced_greedy([(gh, s, 35, 100_000, 7)])
-    tuned, _ = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, 37, 100_000, 7))
-    after, _ = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, 37, 100_000, 7))
+    assert counts[16] > counts[0] and set(counts[:16] + counts[17:]) == {counts[0]}, counts
+    cuda_lib.batch_advanced_greedy([(gh, s, 75, 100_000, 7)])
+    tuned, _ = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, 85, 100_000, 7))
+    after, _ = _launches(cuda_lib, lambda: cuda_lib.advanced_greedy(gh, s, 85, 100_000, 7))
     assert tuned >= after + 2 * TIMED_CALLS, (tuned, after)
-    assert np.array_equal(cuda_lib.estimate_decrease(gh, s, [], 8192, 3, 0), want)
+    assert np.array_equal(cuda_lib.estimate_decrease(gh, s, [], 1000, 3, 0), want)
 
 
 def test_huge_cascades_drop_the_warp_tier_below_1024_samples_a_round(cuda_lib, monkeypatch):
@@ -96,7 +96,7 @@ def test_a_tuned_cutoff_is_shared_by_handles_of_one_graph(cuda_lib):
     assert np.array_equal(d1, want) and np.array_equal(d2, want)
 
 
-@pytest.mark.parametrize("theta,rounds,budget", [(100_000, 71, 5), (7_000, 1001, 4)])
+@pytest.mark.parametrize("theta,rounds,budget", [(100_000, 160, 5), (7_000, 1001, 4)])
 def test_the_tuner_times_the_kernels_of_the_call(cuda_lib, theta, rounds, budget):
     """The warp tier has one instantiation for rounds of more than two samples per resident warp (5 blocks
     per SM) and one for fewer (4); the line lies at 7,296 samples where a cutoff leaves 3 blocks per SM,
@@ -149,8 +149,8 @@ def test_a_costly_warm_up_runs_once_per_graph(cuda_lib):
 
 
 def test_a_first_short_call_runs_its_own_kernels_only(cuda_lib):
-    """Fewer than 16,384 samples over all rounds, in one call of a driver or in the queries of a batch: no
-    warm-up, whose 1,024 samples would be a good part of the call."""
+    """Short rounds, fewer than 16,384 samples over all of them, in one call of a driver or in the queries of
+    a batch: no warm-up, whose 1,024 samples would be a good part of the call."""
     g = _chung_lu(3000, 15000, 571)
     s = W.uniform_seeds(g.n, 10, 572)
     gh = cuda_lib.load_graph(g)
